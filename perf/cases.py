@@ -96,10 +96,10 @@ def _window(case):
     return (None if case["mode"] == "full" else W), theta
 
 
-def prepare(case, seed):
+def _inputs(case, seed):
+    """What the case draws: queries, keys and values before any rotation (a decode's are what its cache holds)."""
     Hq, Hkv, d, _, _ = LAYERS[case["layer"]]
     B, N = case["B"], _length(case)
-    W, theta = _window(case)
     gen = torch.Generator(device="cuda")
     gen.manual_seed(seed)
 
@@ -111,13 +111,30 @@ def prepare(case, seed):
                 out[b, h] = torch.randn(shape[2:], generator=gen, dtype=torch.float32, device="cuda")
         return out
 
-    state = {"case": case, "theta": theta,
-             "table": None if W is None else atf.WindowTable(W),
-             "mode": atf.ATF_MODE_COARSE if case["mode"] == "coarse" else atf.ATF_MODE_EXACT}
     if case["op"] == "decode":
         # keys and values of the context; the query has been rotated by the program
         K = normal((B, Hkv, N, d))
-        state["q"], state["V"] = normal((B, Hq, d)), normal((B, Hkv, N, d))
+        return normal((B, Hq, d)), K, normal((B, Hkv, N, d))
+    kind = torch.float32 if case["op"] == "split" else torch.bfloat16
+    Q, K, V = normal((B, Hq, case.get("Nq", N), d), kind), normal((B, Hkv, N, d), kind), normal((B, Hkv, N, d))
+    if case.get("outlier"):
+        h = d // 2
+        for t in (Q, K):
+            t[..., h - 4:h] *= 8
+            t[..., d - 4:] *= 8
+    return Q, K, V
+
+
+def prepare(case, seed):
+    _, Hkv, d, _, _ = LAYERS[case["layer"]]
+    B, N = case["B"], _length(case)
+    W, theta = _window(case)
+    Q, K, V = _inputs(case, seed)
+    state = {"case": case, "theta": theta, "V": V,
+             "table": None if W is None else atf.WindowTable(W),
+             "mode": atf.ATF_MODE_COARSE if case["mode"] == "coarse" else atf.ATF_MODE_EXACT}
+    if case["op"] == "decode":
+        state["q"] = Q
         if case["cache"] == "rows":
             state["K"] = K
         else:
@@ -126,13 +143,6 @@ def prepare(case, seed):
             if case["cache"] == "unrotated":
                 state["tables"] = atf.atf_rope_tables(theta, d, N + 512)
         return state
-    kind = torch.float32 if case["op"] == "split" else torch.bfloat16
-    Q, K, V = normal((B, Hq, case.get("Nq", N), d), kind), normal((B, Hkv, N, d), kind), normal((B, Hkv, N, d))
-    if case.get("outlier"):
-        h = d // 2
-        for t in (Q, K):
-            t[..., h - 4:h] *= 8
-            t[..., d - 4:] *= 8
     if case["op"] == "layer":
         # fresh projections: the step itself rotates them
         state["cache"] = atf.new_kcache_groups(B, Hkv, N + 512, d, "cuda")
@@ -140,7 +150,7 @@ def prepare(case, seed):
         rope = atf.atf_rope_f32 if case["op"] == "split" else atf.atf_rope
         rope(Q, theta, pos0=N - Q.shape[2])
         rope(K, theta)
-    state["Q"], state["K"], state["V"] = Q, K, V
+    state["Q"], state["K"] = Q, K
     return state
 
 
@@ -203,3 +213,105 @@ def tolerance(case):
     # prompts of 4000 to 8000 tokens: 2.1e-3 (split precision, d = 128) to 2.4e-3 (decode) in the 2-norm, largest element
     # 0.025 of the output's root mean square; LSE 4e-7.  Four times that.
     return {"rel": 9e-3, "max": 0.1}
+
+
+def _frequencies(case):
+    """Angular frequencies and window widths of the layer, from their formulas."""
+    _, _, d, base, scaled = LAYERS[case["layer"]]
+    N, theta, W = _length(case), [], []
+    for r in range(d // 2):
+        f = base ** (-2.0 * r / d)
+        if scaled:  # llama3 rule: factor 32, low 1, high 4, original context 8192
+            lam = 2.0 * math.pi / f
+            if lam > 8192.0:
+                f /= 32.0
+            elif lam >= 8192.0 / 4.0:
+                t = (8192.0 / lam - 1.0) / 3.0
+                f = (1.0 - t) * f / 32.0 + t * f
+        w = K_WINDOW * (2.0 * math.pi / f)
+        theta.append(f)
+        W.append(int(w) if case["mode"] != "full" and w < N else N)
+    if case["mode"] == "coarse":  # groups of eight pairs live as long as their widest window
+        W = [W[r // 8 * 8 + 7] for r in range(d // 2)]
+    return torch.tensor(theta, dtype=torch.float64, device="cuda"), W
+
+
+def _rotated(X, theta, pos0):
+    """Half-split rotation in 64 bits, rounded to what X holds (that is what attention is given)."""
+    h = X.shape[-1] // 2
+    out = torch.empty_like(X)
+    ang = torch.arange(pos0, pos0 + X.shape[-2], dtype=torch.float64, device="cuda")[:, None] * theta
+    c, s = ang.cos(), ang.sin()
+    for b in range(X.shape[0]):
+        for i in range(X.shape[1]):
+            x, y = X[b, i, :, :h].double(), X[b, i, :, h:].double()
+            out[b, i, :, :h], out[b, i, :, h:] = (x * c - y * s).to(X.dtype), (y * c + x * s).to(X.dtype)
+    return out
+
+
+def _attend(Q, K, V, W, n0, coarse):
+    """One (batch, KV head) in 64 bits: rows n0.. of the heads Q [g, Nq, d] on keys K, V [N, d]; O and LSE."""
+    g, Nq, d = Q.shape
+    h, blk = d // 2, 512
+    O = torch.empty((g, Nq, d), dtype=torch.float64, device="cuda")
+    lse = torch.empty((g, Nq), dtype=torch.float64, device="cuda")
+    K, V = K.double(), V.double()
+    a = n0
+    while a < n0 + Nq:
+        b = min(a // blk * blk + blk, n0 + Nq)
+        q = Q[:, a - n0:b - n0].double() / math.sqrt(d)
+        S = torch.full((g, b - a, b), -math.inf, dtype=torch.float64, device="cuda")
+        n = torch.arange(a, b, device="cuda")[:, None]
+        for m0 in range(0, b, blk):
+            m1 = min(m0 + blk, b)
+            m = torch.arange(m0, m1, device="cuda")
+            z = n - m
+            # coarse: what is live is decided for a whole 128 x 128 tile, at its nearest cell
+            tiles = n // 128 - m // 128
+            far = torch.where(tiles > 0, tiles * 128 - 127, 0) if coarse else z
+            lo, hi = int(far.min()), int(far.max())
+            every = [r for r in range(h) if W[r] >= hi]
+            dims = every + [r + h for r in every]
+            s = q[..., dims] @ K[m0:m1][:, dims].T if dims else torch.zeros((g, b - a, m1 - m0), dtype=torch.float64, device="cuda")
+            for r in range(h):
+                if lo <= W[r] < hi:
+                    s += (q[..., [r, r + h]] @ K[m0:m1][:, [r, r + h]].T) * (far <= W[r])
+            S[..., m0:m1] = torch.where((z >= 0) & (far <= max(W)), s, -math.inf)
+        lse[:, a - n0:b - n0] = torch.logsumexp(S, -1)
+        O[:, a - n0:b - n0] = torch.softmax(S, -1) @ V[:b]
+        a = b
+    return O, lse
+
+
+def exact(case, seed):
+    """What run() returns, in 64 bits; None where that would take too long (and for the cache, which is a copy)."""
+    Hq, Hkv, d, _, _ = LAYERS[case["layer"]]
+    B, N, g = case["B"], _length(case), Hq // Hkv
+    Nq = 1 if case["op"] == "decode" else case.get("Nq", N)
+    if B * Hq * (Nq * (N - Nq) + Nq * (Nq + 1) // 2) > 2e10:
+        return None
+    theta, W = _frequencies(case)
+    Q, K, V = _inputs(case, seed)
+    coarse = case["mode"] == "coarse"
+    if case["op"] == "decode":
+        Q = Q[:, :, None]
+        if case["cache"] == "unrotated":
+            K = _rotated(K, theta, 0)
+    else:
+        Q, K = _rotated(Q, theta, N - Nq), _rotated(K, theta, 0)
+
+    def attention(q, n0, tiles):
+        O = torch.empty(q.shape, dtype=torch.float64, device="cuda")
+        lse = torch.empty(q.shape[:3], dtype=torch.float64, device="cuda")
+        for b in range(B):
+            for k in range(Hkv):
+                O[b, k * g:(k + 1) * g], lse[b, k * g:(k + 1) * g] = _attend(q[b, k * g:(k + 1) * g], K[b, k], V[b, k], W, n0, tiles)
+        return O, lse
+
+    if case["op"] == "decode":
+        O, lse = attention(Q, N - 1, False)
+        return O[:, :, 0] if case["cache"] == "rows" else (O[:, :, 0], lse[:, :, 0])
+    O, lse = attention(Q, N - Nq, coarse)
+    if case["op"] == "layer":
+        return O, lse, attention(Q[:, :, -1:], N - 1, False)[0][:, :, 0], None
+    return O, lse
