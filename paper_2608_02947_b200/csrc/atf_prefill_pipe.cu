@@ -118,6 +118,14 @@ __device__ __forceinline__ float exp_half(float (&s)[64], float scale, float neg
   return (a01.x + a01.y) + (a23.x + a23.y);
 }
 
+// C (16 x 8, fp32 fragment) += A (16 x 16) B (16 x 8), bf16.
+__device__ __forceinline__ void mma_16816(float* c, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                          uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
 // Band schedule (Sec. 3.3: the active pairs of a tile are known statically).  What a step needs depends only on
 // the tile distance dt and on which 32 rows x 64 keys of the tile a softmax warp owns (quarter wq of the rows,
 // half h of the keys); it is the same for every CTA of a launch.  A pre-kernel writes one word per (dt, wq, h):
@@ -497,88 +505,96 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         tc_fence_after();
         // S(t) is complete, so Q is not being read: zero what the quarter does not keep in the next tile's MMA
         if (MODE == ATF_MODE_EXACT && t + 1 < nt) zero_q_down_to(p_mid_next);
+        bool s_valid = natoms > 0;  // else no pair is kept in the MMA of this tile and S was not written
+        if (MODE == ATF_MODE_EXACT) {
+          // ---- per-cell finish.  Pairs [p_all, p_mid) went through the MMA and are not live in every cell of
+          //      the warp's block: take their term back out of the cells beyond the window.  Pairs [p_mid, p_any)
+          //      are zero in Q and live somewhere in the block: add their term inside the window.
+          //      One pair's masked term of 16 rows x 8 keys is ONE m16n8k16 product: the contraction runs over
+          //      eight slots of two elements, slot j = key j; B holds the pair of key j in slot j only, A the
+          //      pair of each row in the slots of the keys it takes.  S is brought in and put back in the
+          //      accumulator-fragment order. ----
+          const int p_lo = min(p_all, p_mid), p_hi = max(p_any, p_mid);
+          if (p_lo < p_hi && zmax_w >= 0) {
+            uint32_t q_next = *reinterpret_cast<const uint32_t*>(qsrc + 2 * p_lo), ql_next = 0u;
+            if (SPLIT) ql_next = *reinterpret_cast<const uint32_t*>(qsrc_lo + 2 * p_lo);
+            if (!wait_or_abort(bar(B_KFULL + ks), (g / KS) & 1, abortp)) { ok = false; fail_site = 32; break; }
+            float f[2][32];  // rows 16 hf + {lane / 4, lane / 4 + 8}, keys 64h + 8 cb + 2 (lane % 4) + {0, 1}
+            if (s_valid) {
+              tc_ld_frag64(tS, f[0]);
+              tc_ld_frag64(tS + (16u << 16), f[1]);
+              tc_wait_ld();
+            } else {
+#pragma unroll
+              for (int e = 0; e < 32; ++e) f[0][e] = f[1][e] = 0.f;
+              s_valid = true;
+            }
+            const int g8 = lane >> 2, t4 = lane & 3;
+            const uint32_t slot0 = g8 == t4 ? 0xFFFFFFFFu : 0u, slot4 = g8 == t4 + 4 ? 0xFFFFFFFFu : 0u;
+            const int zw_lo = dt * T + wq * 32, zw_hi = zw_lo + 31;  // zrow over the warp's rows
+            const uint32_t krow = sK + ks * SM::KSTAGE + (64 * h + g8) * 128;
+#pragma unroll 1
+            for (int p = p_lo; p < p_hi; ++p) {
+              const bool subtract = p < p_mid;
+              const uint32_t flip = subtract ? 0x80008000u : 0u;
+              const uint32_t qq = q_next ^ flip, ql = ql_next ^ flip;
+              const int pn = min(p + 1, p_hi - 1);
+              q_next = *reinterpret_cast<const uint32_t*>(qsrc + 2 * pn);
+              if (SPLIT) ql_next = *reinterpret_cast<const uint32_t*>(qsrc_lo + 2 * pn);
+              const int wp = sW[H - 1 - p];
+              uint32_t qr[4], qrl[SPLIT ? 4 : 1];  // the pair of rows g8 + 8 j
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                qr[j] = __shfl_sync(0xffffffffu, qq, g8 + 8 * j);
+                if (SPLIT) qrl[j] = __shfl_sync(0xffffffffu, ql, g8 + 8 * j);
+              }
+              // row g8 + 8 j takes the key of slot t4 (t4 + 4) of block cb inside the window iff 8 (cb - j) >= u (u - 4)
+              const int u = zw_lo + g8 - t4 - 64 * h - wp;
+              const uint32_t kp = krow + ((2 * p) >> 6) * BLK_BYTES + (((((2 * p) & 63) >> 3) ^ g8) << 4) + ((2 * p) & 7) * 2;
+#pragma unroll
+              for (int c2 = 0; c2 < 4; ++c2) {  // 16 keys at a time: distances [zw_lo - c0 - 15, zw_hi - c0]
+                const int c0 = 64 * h + 16 * c2;
+                if (subtract ? zw_hi - c0 > wp : (zw_lo - c0 - 15 <= wp && zw_hi >= c0)) {  // warp-uniform
+#pragma unroll
+                  for (int cb = 2 * c2; cb < 2 * c2 + 2; ++cb) {
+                    uint32_t kk, kl = 0u;
+                    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(kk) : "r"(kp + cb * 1024));
+                    if (SPLIT) asm volatile("ld.shared.b32 %0, [%1];" : "=r"(kl) : "r"(kp + SM::TILE + cb * 1024));
+#pragma unroll
+                    for (int hf = 0; hf < 2; ++hf) {
+                      const int i0 = 8 * (cb - 2 * hf), i1 = i0 - 8;  // rows g8 and g8 + 8 of the half
+                      const bool m0 = (i0 >= u) != subtract, m1 = (i1 >= u) != subtract;
+                      const bool m2 = (i0 + 4 >= u) != subtract, m3 = (i1 + 4 >= u) != subtract;
+                      const uint32_t a0 = m0 ? qr[2 * hf] : 0u, a1 = m1 ? qr[2 * hf + 1] : 0u;
+                      const uint32_t a2 = m2 ? qr[2 * hf] : 0u, a3 = m3 ? qr[2 * hf + 1] : 0u;
+                      mma_16816(f[hf] + 4 * cb, a0, a1, a2, a3, kk & slot0, kk & slot4);
+                      if (SPLIT) {  // the other two products of the split scores
+                        mma_16816(f[hf] + 4 * cb, a0, a1, a2, a3, kl & slot0, kl & slot4);
+                        mma_16816(f[hf] + 4 * cb, m0 ? qrl[2 * hf] : 0u, m1 ? qrl[2 * hf + 1] : 0u, m2 ? qrl[2 * hf] : 0u,
+                                  m3 ? qrl[2 * hf + 1] : 0u, kk & slot0, kk & slot4);
+                      }
+                    }
+                  }
+                }
+              }
+            }
+            tc_st_frag64(tS, f[0]);
+            tc_st_frag64(tS + (16u << 16), f[1]);
+            tc_wait_st();
+          }
+        }
         float s[64];
-        if (natoms > 0) {
+        if (s_valid) {
           tc_ld32(tS, reinterpret_cast<uint32_t*>(s));
           tc_ld32(tS + 32, reinterpret_cast<uint32_t*>(s) + 32);
           tc_wait_ld();
-        } else {  // no pair is kept in the MMA of this tile: every live term is added below
+        } else {
 #pragma unroll
           for (int c = 0; c < 64; ++c) s[c] = 0.f;
         }
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(bar(B_SREAD + sb));
-
-        if (MODE == ATF_MODE_EXACT) {
-          // ---- per-cell finish.  Pairs [p_all, p_mid) went through the MMA and are not live in every cell of
-          //      the warp's block: take their term back out of the cells beyond the window.  Pairs [p_mid, p_any)
-          //      are zero in Q and live somewhere in the block: add their term inside the window.  32 columns at
-          //      a time, skipping what no row of the warp needs. ----
-          const int p_lo = min(p_all, p_mid), p_hi = max(p_any, p_mid);
-          if (p_lo < p_hi && zmax_w >= 0) {
-            if (!wait_or_abort(bar(B_KFULL + ks), (g / KS) & 1, abortp)) { ok = false; fail_site = 32; break; }
-            const int zw_lo = dt * T + wq * 32, zw_hi = zw_lo + 31;  // zrow over the warp's rows
-            for (int p = p_lo; p < p_hi; ++p) {
-              const bool subtract = p < p_mid;
-              if (subtract ? p < p_all : p >= p_any) continue;  // live everywhere and in the MMA / dead everywhere and zeroed
-              const int wp = sW[H - 1 - p];
-              // distances of the warp's cells in columns 64h + 32q .. + 31: [zw_lo - c1, zw_hi - c0]
-              bool touched[2];
-#pragma unroll
-              for (int q = 0; q < 2; ++q) {
-                const int c0 = 64 * h + 32 * q;
-                const int hi = zw_hi - c0, lo = zw_lo - c0 - 31;
-                touched[q] = subtract ? (hi > wp) : (lo <= wp && hi >= 0);
-              }
-              if (!touched[0] && !touched[1]) continue;
-              // q0, q1: the pair's two elements of this row (hi parts in the split mode); qs0, qs1: hi + lo there
-              // (exact in fp32: 16 significant bits), so that the term below is the three products of the MMA
-              const uint32_t qq = *reinterpret_cast<const uint32_t*>(qsrc + 2 * p);
-              float q0 = bf16lo_to_f32(qq), q1 = bf16hi_to_f32(qq);
-              float qs0 = q0, qs1 = q1;
-              if (SPLIT) {
-                const uint32_t ql = *reinterpret_cast<const uint32_t*>(qsrc_lo + 2 * p);
-                qs0 += bf16lo_to_f32(ql);
-                qs1 += bf16hi_to_f32(ql);
-              }
-              if (subtract) {
-                q0 = -q0;
-                q1 = -q1;
-                qs0 = -qs0;
-                qs1 = -qs1;
-              }
-              const int col = 2 * p;
-              const uint32_t kb32 = sK + ks * SM::KSTAGE + (col >> 6) * BLK_BYTES + (col & 7) * 2;
-              const int chunk = (col & 63) >> 3;
-              // cells with column >= jb = zrow - w are inside the window: adding uses sat(c - jb + 1), taking back
-              // sat(jb - c), formed on the FMA pipe
-              const float jbf = (float)(zrow - wp - 64 * h);
-              const float ca = subtract ? -1.f : 1.f, cb = subtract ? jbf : 1.f - jbf;
-#pragma unroll
-              for (int q = 0; q < 2; ++q) {
-                if (touched[q]) {  // warp-uniform
-                  uint32_t kk[32], kl[SPLIT ? 32 : 1];
-#pragma unroll
-                  for (int cc = 0; cc < 32; ++cc) {
-                    const int c = 64 * h + 32 * q + cc;  // key of the tile; (c & 7) does not depend on h
-                    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(kk[cc]) : "r"(kb32 + ((chunk ^ (c & 7)) << 4) + c * 128));
-                    if (SPLIT)
-                      asm volatile("ld.shared.b32 %0, [%1];" : "=r"(kl[cc]) : "r"(kb32 + SM::TILE + ((chunk ^ (c & 7)) << 4) + c * 128));
-                  }
-#pragma unroll
-                  for (int cc = 0; cc < 32; ++cc) {
-                    const int cl = 32 * q + cc;  // column of this thread's half
-                    float term = fmaf(qs0, bf16lo_to_f32(kk[cc]), qs1 * bf16hi_to_f32(kk[cc]));
-                    if (SPLIT) term = fmaf(q0, bf16lo_to_f32(kl[cc]), fmaf(q1, bf16hi_to_f32(kl[cc]), term));
-                    const float coef = __saturatef(fmaf(ca, (float)cl, cb));
-                    s[cl] = fmaf(term, coef, s[cl]);
-                  }
-                }
-              }
-            }
-          }
-        }
         // ---- causal mask on the diagonal tile, dropped keys (exact mode: no pair reaches the cell) ----
         if (dt == 0 || (MODE == ATF_MODE_EXACT && zmax_w > Wmax)) {
           const int zdrop = MODE == ATF_MODE_EXACT ? Wmax : 0x7FFFFFFF;
