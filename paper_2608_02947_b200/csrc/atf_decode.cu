@@ -91,6 +91,68 @@ __device__ __forceinline__ float ex2f(float x) {
   return y;
 }
 
+// The last block of a (batch, KV head) merges the partials of all splits by their log-sum-exp: one warp per head.  What
+// this costs is round trips to L2, so every load that can be in flight is: the (m, l) of up to 128 splits in one round
+// (lanes across the splits), then the outputs of MERGE_BATCH splits a round (lanes across the columns; past the last
+// split the loads repeat it with weight 0, because a remainder loop would pay a round trip for each split).
+constexpr int MERGE_BATCH = 16;
+template <int D, int NWARPS>
+__device__ __forceinline__ void merge_splits(const DecodeParams& P, int64_t grp, int64_t hq0, int warp, int lane) {
+  constexpr int PSTRIDE = D + 2;
+  const int G = P.G, ns = P.nsplit;
+  const float* allp = P.partials + grp * ns * (int64_t)(G * PSTRIDE);
+  for (int gg = warp; gg < G; gg += NWARPS) {
+    const float* base = allp + (int64_t)gg * PSTRIDE;
+    const int64_t step = (int64_t)G * PSTRIDE;  // floats between two splits
+    float M = -INFINITY, L = 0.f;                // of this lane's splits
+    for (int s0 = lane; s0 < ns; s0 += 128) {
+      float m[4], l[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const bool in = s0 + 32 * i < ns;
+        m[i] = in ? __ldcg(base + (s0 + 32 * i) * step) : -INFINITY;
+        l[i] = in ? __ldcg(base + (s0 + 32 * i) * step + 1) : 0.f;
+      }
+      const float mx = fmaxf(fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3])), M), ms = mx == -INFINITY ? 0.f : mx;
+      L *= ex2f(M - ms);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) L += ex2f(m[i] - ms) * l[i];
+      M = mx;
+    }
+    float Ms = M;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) Ms = fmaxf(Ms, __shfl_xor_sync(0xffffffffu, Ms, off));
+    if (Ms == -INFINITY) Ms = 0.f;
+    L *= ex2f(M - Ms);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) L += __shfl_xor_sync(0xffffffffu, L, off);
+    float acc[D / 32];
+#pragma unroll
+    for (int c = 0; c < D / 32; ++c) acc[c] = 0.f;
+    for (int s0 = 0; s0 < ns; s0 += MERGE_BATCH) {
+      float f[MERGE_BATCH], o[MERGE_BATCH][D / 32];
+#pragma unroll
+      for (int i = 0; i < MERGE_BATCH; ++i) {
+        const float* src = base + min(s0 + i, ns - 1) * step;
+        f[i] = __ldcg(src);
+#pragma unroll
+        for (int c = 0; c < D / 32; ++c) o[i][c] = __ldcg(src + 2 + c * 32 + lane);
+      }
+#pragma unroll
+      for (int i = 0; i < MERGE_BATCH; ++i) {
+        const float w = s0 + i < ns ? ex2f(f[i] - Ms) : 0.f;
+#pragma unroll
+        for (int c = 0; c < D / 32; ++c) acc[c] = fmaf(w, o[i][c], acc[c]);
+      }
+    }
+    const float inv = 1.f / L;
+    const int64_t hq = hq0 + gg;
+#pragma unroll
+    for (int c = 0; c < D / 32; ++c) P.O[hq * D + c * 32 + lane] = __float2bfloat16_rn(acc[c] * inv);
+    if (P.lse && lane == 0) P.lse[hq] = (Ms + log2f(L)) * 0.6931471805599453f;
+  }
+}
+
 template <int D, int MODE, bool COUNT>
 __global__ void __launch_bounds__(DEC_THREADS, 2)
 atf_decode_kernel(const __grid_constant__ DecodeParams P, const __grid_constant__ AtfTable table) {
@@ -423,37 +485,7 @@ atf_decode_kernel(const __grid_constant__ DecodeParams P, const __grid_constant_
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  const float* allp = P.partials + grp * P.nsplit * (int64_t)(G * PSTRIDE);
-  // one warp per head: lanes stride over the splits for the LSE merge, then over columns
-  for (int gg = warp; gg < G; gg += DEC_WARPS) {
-    float M = -INFINITY;
-    for (int sp = lane; sp < P.nsplit; sp += 32) M = fmaxf(M, __ldcg(allp + ((int64_t)sp * G + gg) * PSTRIDE));
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, off));
-    const float Ms = (M == -INFINITY) ? 0.f : M;
-    float Lsum = 0.f;
-    for (int sp = lane; sp < P.nsplit; sp += 32) {
-      const float* src = allp + ((int64_t)sp * G + gg) * PSTRIDE;
-      Lsum += ex2f(__ldcg(src) - Ms) * __ldcg(src + 1);
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) Lsum += __shfl_xor_sync(0xffffffffu, Lsum, off);
-    const float inv = 1.f / Lsum;
-    float acc[D / 32];
-#pragma unroll
-    for (int c = 0; c < D / 32; ++c) acc[c] = 0.f;
-#pragma unroll 8
-    for (int sp = 0; sp < P.nsplit; ++sp) {
-      const float* src = allp + ((int64_t)sp * G + gg) * PSTRIDE;
-      const float f = ex2f(__ldcg(src) - Ms);
-#pragma unroll
-      for (int c = 0; c < D / 32; ++c) acc[c] = fmaf(f, __ldcg(src + 2 + c * 32 + lane), acc[c]);
-    }
-    const int64_t hq = (int64_t)b * P.Hq + hkv * G + gg;
-#pragma unroll
-    for (int c = 0; c < D / 32; ++c) P.O[hq * D + c * 32 + lane] = __float2bfloat16_rn(acc[c] * inv);
-    if (P.lse && lane == 0) P.lse[hq] = (Ms + log2f(Lsum)) * 0.6931471805599453f;
-  }
+  merge_splits<D, DEC_WARPS>(P, grp, (int64_t)b * P.Hq + hkv * G, warp, lane);
   if (threadIdx.x == 0) P.counters[grp] = 0;  // ready for the next launch
 }
 
@@ -834,36 +866,7 @@ atf_decode_tiles_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_co
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  const float* allp = P.partials + grp * P.nsplit * (int64_t)(G * PSTRIDE);
-  for (int gg = warp; gg < G; gg += DEC_WARPS + 1) {
-    float M = -INFINITY;
-    for (int sp = lane; sp < P.nsplit; sp += 32) M = fmaxf(M, __ldcg(allp + ((int64_t)sp * G + gg) * PSTRIDE));
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, off));
-    const float Ms = (M == -INFINITY) ? 0.f : M;
-    float Lsum = 0.f;
-    for (int sp = lane; sp < P.nsplit; sp += 32) {
-      const float* src = allp + ((int64_t)sp * G + gg) * PSTRIDE;
-      Lsum += ex2f(__ldcg(src) - Ms) * __ldcg(src + 1);
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) Lsum += __shfl_xor_sync(0xffffffffu, Lsum, off);
-    const float inv = 1.f / Lsum;
-    float acc[D / 32];
-#pragma unroll
-    for (int c = 0; c < D / 32; ++c) acc[c] = 0.f;
-#pragma unroll 8
-    for (int sp = 0; sp < P.nsplit; ++sp) {
-      const float* src = allp + ((int64_t)sp * G + gg) * PSTRIDE;
-      const float f = ex2f(__ldcg(src) - Ms);
-#pragma unroll
-      for (int c = 0; c < D / 32; ++c) acc[c] = fmaf(f, __ldcg(src + 2 + c * 32 + lane), acc[c]);
-    }
-    const int64_t hq = (int64_t)b * P.Hq + hkv * G + gg;
-#pragma unroll
-    for (int c = 0; c < D / 32; ++c) P.O[hq * D + c * 32 + lane] = __float2bfloat16_rn(acc[c] * inv);
-    if (P.lse && lane == 0) P.lse[hq] = (Ms + log2f(Lsum)) * 0.6931471805599453f;
-  }
+  merge_splits<D, DEC_WARPS + 1>(P, grp, (int64_t)b * P.Hq + hkv * G, warp, lane);
   if (threadIdx.x == 0) P.counters[grp] = 0;  // ready for the next launch
 }
 
@@ -944,14 +947,45 @@ atf_status launch_decode_tiles(const CUtensorMap& tmV, const DecodeParams& P, co
 
 atf_status atf_validate_table(const char* who, const int64_t* table, int d, int64_t N, AtfTable* out);
 
-static size_t decode_ws_bytes(int B, int Hq, int Hkv, int64_t L, int d) {
-  const int ns = std::max(atf_decode_num_splits(B, Hkv, L, ATF_DECODE_SLOTS_ROWS),
-                          atf_decode_num_splits(B, Hkv, L, ATF_DECODE_SLOTS_GROUPS));
+// Splits of a (batch, KV head) over which a launch deals its `ntiles` tiles.  In units of one tile of a CTA that shares
+// its SM with another (about 1 us; alone on the SM it takes 3/4 of that), a launch costs
+//   the tiles a CTA walks, for each round of CTAs an SM runs (two at a time), + 14 for every round after the first
+//   (prologue, first loads, partials: 240 us in one round against 246 in two and 289 in four, eight sequences of 128K)
+//   + the merge: a round trip to L2 for every MERGE_BATCH splits and every DEC_WARPS heads.
+// Measured, d = 128, 24/8 heads, the rule this replaced (at least 512 keys a split, fullest last wave) -> this one:
+// 512 keys 18.7 -> 8.2 us, 2048 keys 18.0 -> 10.2, 4096 keys 17.7 -> 12.6; two sequences of 32K 63 -> 50 us, eight
+// 151 -> 128 us.  Of equal costs the fewest splits are taken.
+static int decode_splits(int64_t groups, int heads, int64_t ntiles) {
+  constexpr int SMS = 148;
+  const int64_t most = std::min<int64_t>(ntiles, std::max<int64_t>(1, 4 * SMS / groups));
+  double best = 0.0;
+  int best_ns = 0;
+  for (int64_t ns = 1; ns <= most; ++ns) {
+    const int64_t per_sm = (groups * ns + SMS - 1) / SMS;
+    const double tiles = (double)((ntiles + ns - 1) / ns);
+    const double cost = tiles * ((double)(per_sm / 2) + 0.75 * (double)(per_sm & 1)) + 14.0 * (double)((per_sm - 1) / 2) +
+                        (double)((ns + MERGE_BATCH - 1) / MERGE_BATCH * ((heads + DEC_WARPS - 1) / DEC_WARPS));
+    if (best_ns == 0 || cost < best) {
+      best = cost;
+      best_ns = (int)ns;
+    }
+  }
+  return best_ns;
+}
+
+// The least scratch a call is taken with (fewer splits than decode_splits asks for where it holds no more).
+static size_t decode_ws_least(int B, int Hq, int Hkv, int64_t L, int d) {
+  static_assert(ATF_DECODE_SLOTS_ROWS == ATF_DECODE_SLOTS_GROUPS, "one count serves both layouts");
+  const int ns = atf_decode_num_splits(B, Hkv, L, ATF_DECODE_SLOTS_ROWS);
   size_t partials = (size_t)B * Hq * ns * (d + 2) * sizeof(float);
   partials = (partials + 255) & ~(size_t)255;
   return ATF_WS_HEADER + partials;
 }
-size_t atf_decode_workspace_bytes(int B, int Hq, int Hkv, int64_t L, int d) { return decode_ws_bytes(B, Hq, Hkv, L, d); }
+size_t atf_decode_workspace_bytes(int B, int Hq, int Hkv, int64_t L, int d) {
+  const int64_t kt = DEC_WARPS * (DEC_TILE_BYTES / (d * 2));
+  const size_t partials = (size_t)B * Hq * decode_splits((int64_t)B * Hkv, std::max(1, Hq / Hkv), (L + kt - 1) / kt) * (d + 2) * sizeof(float);
+  return std::max(decode_ws_least(B, Hq, Hkv, L, d), ATF_WS_HEADER + ((partials + 255) & ~(size_t)255));
+}
 
 extern "C" atf_status atf_decode_ex(const void* q, const void* Kcache, const void* Vcache, void* O, int B, int Hq,
                                     int Hkv, int64_t L, int d, const int64_t* table, const atf_opts* opts,
@@ -974,7 +1008,7 @@ extern "C" atf_status atf_decode_ex(const void* q, const void* Kcache, const voi
 
   AtfWorkspace ws = atf_bound_workspace();
   if (opts && opts->workspace) ws = AtfWorkspace{opts->workspace, opts->workspace_bytes};
-  const size_t need = decode_ws_bytes(B, Hq, Hkv, L, d);
+  const size_t need = decode_ws_least(B, Hq, Hkv, L, d);
   if (!ws.ptr) return atf_fail(ATF_ERR_WORKSPACE, "atf_decode: no workspace bound");
   if (ws.bytes < need) return atf_fail(ATF_ERR_WORKSPACE, "atf_decode: workspace has %zu bytes, needs %zu", ws.bytes, need);
   if ((uintptr_t)ws.ptr & 255) return atf_fail(ATF_ERR_INVALID_ARG, "atf_decode: workspace must be 256-byte aligned");
@@ -991,10 +1025,10 @@ extern "C" atf_status atf_decode_ex(const void* q, const void* Kcache, const voi
   P.G = Hq / Hkv;
   P.L = (int)L;
   const int kl_ = opts ? opts->k_layout : ATF_KLAYOUT_ROWS;
-  P.nsplit = atf_decode_num_splits(B, Hkv, L, kl_ == ATF_KLAYOUT_GROUPS ? ATF_DECODE_SLOTS_GROUPS : ATF_DECODE_SLOTS_ROWS);
   const int64_t kt = DEC_WARPS * (DEC_TILE_BYTES / (d * 2));  // keys per tile; tiles go round-robin to the splits
   const int64_t ntiles = (L + kt - 1) / kt;
-  if (P.nsplit > ntiles) P.nsplit = (int)ntiles;
+  const int64_t fit = (int64_t)((ws.bytes - ATF_WS_HEADER) / ((size_t)B * Hq * (d + 2) * sizeof(float)));  // >= 1
+  P.nsplit = (int)std::min<int64_t>(decode_splits((int64_t)B * Hkv, P.G, ntiles), fit);
   // a group-major cache laid out for more keys than it holds yet (room for the tokens to come)
   const int64_t cap = (opts && opts->kcache_capacity > 0) ? opts->kcache_capacity : L;
   if (cap < L) return atf_fail(ATF_ERR_INVALID_ARG, "atf_decode: kcache_capacity (%lld) is smaller than L", (long long)cap);
@@ -1138,7 +1172,7 @@ extern "C" atf_status atf_decode_static(const void* q, const void* Kcache, const
   if (B < 1 || Hq < 1 || Hkv < 1 || L < 1 || (d != 64 && d != 128) || Hq % Hkv)
     return atf_fail(ATF_ERR_INVALID_ARG, "atf_decode_static: bad shape");
   if ((int64_t)B * Hkv > ATF_WS_COUNTER_SLOTS) return atf_fail(ATF_ERR_UNSUPPORTED, "atf_decode_static: B*Hkv must be <= %d", ATF_WS_COUNTER_SLOTS);
-  const size_t need = decode_ws_bytes(B, Hq, Hkv, L, d);
+  const size_t need = decode_ws_least(B, Hq, Hkv, L, d);
   if (need > ATF_STATIC_SCRATCH_BYTES)
     return atf_fail(ATF_ERR_WORKSPACE,
                     "atf_decode_static: this problem needs %zu bytes of scratch, the built-in array holds %zu; "

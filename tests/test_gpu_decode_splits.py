@@ -1,0 +1,61 @@
+"""Decode: the number of splits of a call, at the sizes where the deal of tiles to splits and the merge can go wrong (one
+tile, one key over a tile, a last split with fewer tiles, more splits than a merge batch), and with scratch for one."""
+import ctypes as C
+
+import numpy as np
+import pytest
+import torch
+
+import atf_inputs as gen
+from oracle import atf_oracle as orc
+
+pytestmark = pytest.mark.gpu
+HEADER = 256 + 16384 * 4  # status words and split counters
+
+
+def _case(B, Hq, Hkv, d, L, seed):
+    w = gen.Workload("splits", B, Hq, Hkv, d, L, 5e5, 2.0, gen.LLAMA3_SCALING, gen.SEED0 + seed)
+    q, K, V = gen.decode_inputs(w)
+    Wo, _ = orc.window_table(w.base, w.d, w.k, w.N, w.scaling)
+    return q, K, V, Wo
+
+
+def _check(O, lse, ref):
+    # P and O are rounded to bf16 (2^-9 each): the tolerances of the other decode tests
+    err = np.abs(gen.to_f64(O) - ref[0])
+    assert err.max() <= 2e-2 and err.mean() <= 2e-3
+    if lse is not None:
+        assert np.abs(lse.double().cpu().numpy() - ref[1]).max() <= 1e-3
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,d,L", [(1, 3, 1, 128, 1), (1, 3, 1, 128, 64), (1, 24, 8, 128, 65), (1, 24, 8, 128, 1023),
+                                          (2, 24, 8, 128, 2113), (1, 14, 2, 64, 129), (1, 14, 2, 64, 1000), (1, 8, 1, 64, 20000),
+                                          (1, 7, 1, 128, 9000), (40, 8, 8, 64, 300)])
+def test_splits_against_oracle(B, Hq, Hkv, d, L):
+    import paper_2608_02947_b200 as atf
+    q, K, V, W = _case(B, Hq, Hkv, d, L, 800 + L)
+    ref = orc.decode(gen.to_f64(q), gen.to_f64(K), gen.to_f64(V), W)
+    q, K, V = q.cuda(), K.cuda(), V.cuda()
+    for cache in (K, atf.atf_kcache_pack(K)):
+        _check(*atf.atf_decode(q, cache, V, table=W, return_lse=True), ref)
+
+
+def test_scratch_for_one_split():
+    import paper_2608_02947_b200 as atf
+    lib = atf.lib()
+    B, Hq, Hkv, d, L = 1, 24, 8, 128, 1000
+    q, K, V, W = _case(B, Hq, Hkv, d, L, 77)
+    ref = orc.decode(gen.to_f64(q), gen.to_f64(K), gen.to_f64(V), W)
+    q, K, V = q.cuda(), K.cuda(), V.cuda()
+    one = HEADER + (Hq * (d + 2) * 4 + 255) // 256 * 256
+    assert lib.atf_workspace_bytes(1, B, Hq, Hkv, L, d) > one
+    ws = torch.zeros(one, dtype=torch.uint8, device="cuda")
+    O = torch.empty_like(q)
+    tab = (C.c_int64 * (d // 2))(*[int(x) for x in W])
+    opts = atf.binding._Opts()
+    for nbytes, code in ((one, 0), (one - 256, 4)):
+        opts.workspace, opts.workspace_bytes = ws.data_ptr(), nbytes
+        p = [C.c_void_p(t.data_ptr()) for t in (q, K, V, O)]
+        assert lib.atf_decode_ex(*p, B, Hq, Hkv, L, d, tab, C.byref(opts), C.c_void_p(torch.cuda.current_stream().cuda_stream)) == code
+    torch.cuda.synchronize()
+    _check(O, None, ref)
