@@ -7,134 +7,133 @@ struct RopeTheta {
   double t[ATF_MAX_PAIRS];
 };
 
-// One thread owns 8 consecutive pairs of one row (two 16-byte segments, one per half) and
-// walks over the heads assigned to its blockIdx.y, so sincos is evaluated once per (row, pair).
-template <int D>
-__global__ void __launch_bounds__(256) atf_rope_kernel(__nv_bfloat16* __restrict__ X, int BH, int64_t N, int64_t pos0,
-                                                        const __grid_constant__ RopeTheta theta) {
-  constexpr int H = D / 2;
-  constexpr int CHUNKS = H / 8;  // 16-byte chunks per half row
-  const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t n = gid / CHUNKS;
-  const int c = (int)(gid % CHUNKS);
-  if (n >= N) return;
-  double cs[8], sn[8];
-  const double pos = (double)(pos0 + n);
+// Eight consecutive elements of a row as fp64, and back with one rounding.
+__device__ __forceinline__ void load8(const __nv_bfloat16* p, float (&v)[8]) {
+  const uint4 w = *reinterpret_cast<const uint4*>(p);
+  const uint32_t u[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
-  for (int i = 0; i < 8; ++i) sincos(pos * theta.t[c * 8 + i], &sn[i], &cs[i]);
-  for (int bh = blockIdx.y; bh < BH; bh += gridDim.y) {
-    __nv_bfloat16* row = X + ((int64_t)bh * N + n) * D;
-    uint4 lo = *reinterpret_cast<const uint4*>(row + c * 8);
-    uint4 hi = *reinterpret_cast<const uint4*>(row + H + c * 8);
-    const __nv_bfloat16* lp = reinterpret_cast<const __nv_bfloat16*>(&lo);
-    const __nv_bfloat16* hp = reinterpret_cast<const __nv_bfloat16*>(&hi);
-    uint4 olo, ohi;
-    __nv_bfloat16* ol = reinterpret_cast<__nv_bfloat16*>(&olo);
-    __nv_bfloat16* oh = reinterpret_cast<__nv_bfloat16*>(&ohi);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const double a = (double)__bfloat162float(lp[i]);
-      const double b = (double)__bfloat162float(hp[i]);
-      ol[i] = __double2bfloat16(a * cs[i] - b * sn[i]);
-      oh[i] = __double2bfloat16(b * cs[i] + a * sn[i]);
-    }
-    *reinterpret_cast<uint4*>(row + c * 8) = olo;
-    *reinterpret_cast<uint4*>(row + H + c * 8) = ohi;
+  for (int i = 0; i < 4; ++i) {
+    v[2 * i] = bf16lo_to_f32(u[i]);
+    v[2 * i + 1] = bf16hi_to_f32(u[i]);
   }
 }
-
-// The same rotation on fp32 rows, result kept in fp32 (one rounding from the fp64 rotation): the input of the
-// split-precision prefill, whose point is that the rotated values are never rounded to bf16.
-template <int D>
-__global__ void __launch_bounds__(256) atf_rope_f32_kernel(float* __restrict__ X, int BH, int64_t N, int64_t pos0,
-                                                            const __grid_constant__ RopeTheta theta) {
-  constexpr int H = D / 2;
-  constexpr int CHUNKS = H / 8;
-  const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t n = gid / CHUNKS;
-  const int c = (int)(gid % CHUNKS);
-  if (n >= N) return;
-  double cs[8], sn[8];
-  const double pos = (double)(pos0 + n);
+__device__ __forceinline__ void load8(const float* p, float (&v)[8]) {
+  *reinterpret_cast<float4*>(v) = *reinterpret_cast<const float4*>(p);
+  *reinterpret_cast<float4*>(v + 4) = *reinterpret_cast<const float4*>(p + 4);
+}
+__device__ __forceinline__ void store8(__nv_bfloat16* p, const double (&v)[8]) {
+  uint4 w;
+  __nv_bfloat16* o = reinterpret_cast<__nv_bfloat16*>(&w);
 #pragma unroll
-  for (int i = 0; i < 8; ++i) sincos(pos * theta.t[c * 8 + i], &sn[i], &cs[i]);
-  for (int bh = blockIdx.y; bh < BH; bh += gridDim.y) {
-    float* row = X + ((int64_t)bh * N + n) * D;
-    float lo[8], hi[8];
-    *reinterpret_cast<float4*>(lo) = *reinterpret_cast<const float4*>(row + c * 8);
-    *reinterpret_cast<float4*>(lo + 4) = *reinterpret_cast<const float4*>(row + c * 8 + 4);
-    *reinterpret_cast<float4*>(hi) = *reinterpret_cast<const float4*>(row + H + c * 8);
-    *reinterpret_cast<float4*>(hi + 4) = *reinterpret_cast<const float4*>(row + H + c * 8 + 4);
-    float olo[8], ohi[8];
+  for (int i = 0; i < 8; ++i) o[i] = __double2bfloat16(v[i]);
+  *reinterpret_cast<uint4*>(p) = w;
+}
+__device__ __forceinline__ void store8(float* p, const double (&v)[8]) {
+  float o[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) o[i] = (float)v[i];
+  *reinterpret_cast<float4*>(p) = *reinterpret_cast<const float4*>(o);
+  *reinterpret_cast<float4*>(p + 4) = *reinterpret_cast<const float4*>(o + 4);
+}
+
+// In place, X bf16 or (for the split-precision prefill, whose point is that the rotated values are never rounded to
+// bf16) fp32.  A block owns a few rows of every head and HL threads walk the heads of a row segment (eight pairs: 16
+// bytes of each half row), every HL-th each.  The angles of a segment are evaluated once, in fp64: by its thread (HL = 1)
+// or spread over the block's threads into shared memory.  For long rows memory bounds the pass (24 heads x 131072 x
+// 128: 276 us, 5.8 TB/s).  For short ones HL fills the GPU; spreading the heads over blocks instead, each with the
+// angles evaluated again, made the fp64 pipe the bound: 24 heads x 8192 x 128 23.2 -> 18.0 us, 8 heads 15.3 -> 8.5 us,
+// 24 heads x 2048 12.8 -> 7.1 us.
+constexpr int ROPE_THREADS = 256;
+template <int D, int HL, typename T>
+__global__ void __launch_bounds__(ROPE_THREADS) atf_rope_kernel(T* __restrict__ X, int BH, int64_t N, int64_t pos0,
+                                                                const __grid_constant__ RopeTheta theta) {
+  constexpr int H = D / 2;
+  constexpr int CHUNKS = H / 8;                         // segments of 8 pairs per row
+  constexpr int SEGS = ROPE_THREADS / HL;               // (row, segment) pairs of the block
+  constexpr int ROWS = SEGS / CHUNKS;
+  const int64_t row0 = (int64_t)blockIdx.x * ROWS;
+  const int sg = threadIdx.x % SEGS, c = sg % CHUNKS;
+  const int64_t n = row0 + sg / CHUNKS;
+  double cs[8], sn[8];
+  if constexpr (HL == 1) {  // every thread has a segment of its own: no detour
+    if (n >= N) return;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) sincos((double)(pos0 + n) * theta.t[c * 8 + i], &sn[i], &cs[i]);
+  } else {
+    __shared__ double2 cs_sh[8 * SEGS];  // (cos, sin) of pair i of segment s at i * SEGS + s
+#pragma unroll 1
+    for (int k = threadIdx.x; k < 8 * SEGS; k += ROPE_THREADS) {
+      const int i = k / SEGS, s = k % SEGS;
+      double2 v;
+      sincos((double)(pos0 + row0 + s / CHUNKS) * theta.t[(s % CHUNKS) * 8 + i], &v.y, &v.x);
+      cs_sh[k] = v;
+    }
+    __syncthreads();
+    if (n >= N) return;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const double2 v = cs_sh[i * SEGS + sg];
+      cs[i] = v.x;
+      sn[i] = v.y;
+    }
+  }
+  auto rotate = [&](T* row, const float (&lo)[8], const float (&hi)[8]) {
+    double olo[8], ohi[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const double a = (double)lo[i], b = (double)hi[i];
-      olo[i] = (float)(a * cs[i] - b * sn[i]);
-      ohi[i] = (float)(b * cs[i] + a * sn[i]);
+      olo[i] = a * cs[i] - b * sn[i];
+      ohi[i] = b * cs[i] + a * sn[i];
     }
-    *reinterpret_cast<float4*>(row + c * 8) = *reinterpret_cast<const float4*>(olo);
-    *reinterpret_cast<float4*>(row + c * 8 + 4) = *reinterpret_cast<const float4*>(olo + 4);
-    *reinterpret_cast<float4*>(row + H + c * 8) = *reinterpret_cast<const float4*>(ohi);
-    *reinterpret_cast<float4*>(row + H + c * 8 + 4) = *reinterpret_cast<const float4*>(ohi + 4);
+    store8(row, olo);
+    store8(row + H, ohi);
+  };
+  const int64_t head = N * D;
+  T* row = X + ((int64_t)(threadIdx.x / SEGS) * N + n) * D + c * 8;
+  for (int bh = threadIdx.x / SEGS; bh < BH; bh += HL, row += HL * head) {
+    float lo[8], hi[8];
+    load8(row, lo);
+    load8(row + H, hi);
+    rotate(row, lo, hi);
   }
 }
 
-static atf_status rope_check(const char* who, const void* X, const double* theta, int B, int H, int64_t N, int d,
-                             int64_t pos0) {
+// Threads per row segment: one as long as that gives four blocks (fp32: eight, its rows are twice as long) for each SM, more
+// for shorter rows.
+template <int D, typename T>
+static void launch_rope(T* X, int BH, int64_t N, int64_t pos0, const RopeTheta& th, cudaStream_t s) {
+  int hl = 1;
+  const auto blocks = [&](int lanes) { return (N + ROPE_THREADS / lanes / (D / 16) - 1) / (ROPE_THREADS / lanes / (D / 16)); };
+  while (hl < 8 && blocks(hl) < 2 * (int)sizeof(T) * 148) hl *= 2;
+  const unsigned g = (unsigned)blocks(hl);
+  if (hl == 1) atf_rope_kernel<D, 1, T><<<g, ROPE_THREADS, 0, s>>>(X, BH, N, pos0, th);
+  else if (hl == 2) atf_rope_kernel<D, 2, T><<<g, ROPE_THREADS, 0, s>>>(X, BH, N, pos0, th);
+  else if (hl == 4) atf_rope_kernel<D, 4, T><<<g, ROPE_THREADS, 0, s>>>(X, BH, N, pos0, th);
+  else atf_rope_kernel<D, 8, T><<<g, ROPE_THREADS, 0, s>>>(X, BH, N, pos0, th);
+}
+
+template <typename T>
+static atf_status rope(const char* who, T* X, int B, int H, int64_t N, int d, const double* theta, int64_t pos0, void* stream) {
   if (!X || !theta) return atf_fail(ATF_ERR_INVALID_ARG, "%s: null pointer", who);
   if (d != 64 && d != 128) return atf_fail(ATF_ERR_UNSUPPORTED, "%s: d must be 64 or 128 (got %d)", who, d);
   if (B < 1 || H < 1 || N < 1 || pos0 < 0) return atf_fail(ATF_ERR_INVALID_ARG, "%s: bad shape", who);
   if ((uintptr_t)X & 15) return atf_fail(ATF_ERR_INVALID_ARG, "%s: X must be 16-byte aligned", who);
-  return ATF_OK;
-}
-
-extern "C" atf_status atf_rope_f32(float* X, int B, int H, int64_t N, int d, const double* theta, int64_t pos0,
-                                   void* stream) {
-  atf_status st = rope_check("atf_rope_f32", X, theta, B, H, N, d, pos0);
-  if (st != ATF_OK) return st;
   RopeTheta th;
   for (int r = 0; r < d / 2; ++r) th.t[r] = theta[r];
   for (int r = d / 2; r < ATF_MAX_PAIRS; ++r) th.t[r] = 0.0;
-  const int64_t threads = N * (d / 16);
-  const int64_t blocks = (threads + 255) / 256;
-  if (blocks > 0x7FFFFFFF) return atf_fail(ATF_ERR_UNSUPPORTED, "atf_rope_f32: N too large");
-  const int BH = B * H;
-  int gy = 1;
-  while (gy < BH && blocks * gy < 148 * 8) gy *= 2;
-  if (gy > BH) gy = BH;
-  dim3 grid((unsigned)blocks, (unsigned)gy);
-  cudaStream_t s = (cudaStream_t)stream;
+  if ((N * (d / 16) + 255) / 256 > 0x7FFFFFFF) return atf_fail(ATF_ERR_UNSUPPORTED, "%s: N too large", who);
   if (d == 64)
-    atf_rope_f32_kernel<64><<<grid, 256, 0, s>>>(X, BH, N, pos0, th);
+    launch_rope<64>(X, B * H, N, pos0, th, (cudaStream_t)stream);
   else
-    atf_rope_f32_kernel<128><<<grid, 256, 0, s>>>(X, BH, N, pos0, th);
+    launch_rope<128>(X, B * H, N, pos0, th, (cudaStream_t)stream);
   ATF_CUDA_CHECK(cudaGetLastError());
   return ATF_OK;
 }
 
-extern "C" atf_status atf_rope(void* X, int B, int H, int64_t N, int d, const double* theta, int64_t pos0,
-                               void* stream) {
-  if (!X || !theta) return atf_fail(ATF_ERR_INVALID_ARG, "atf_rope: null pointer");
-  if (d != 64 && d != 128) return atf_fail(ATF_ERR_UNSUPPORTED, "atf_rope: d must be 64 or 128 (got %d)", d);
-  if (B < 1 || H < 1 || N < 1 || pos0 < 0) return atf_fail(ATF_ERR_INVALID_ARG, "atf_rope: bad shape");
-  if ((uintptr_t)X & 15) return atf_fail(ATF_ERR_INVALID_ARG, "atf_rope: X must be 16-byte aligned");
-  RopeTheta th;
-  for (int r = 0; r < d / 2; ++r) th.t[r] = theta[r];
-  for (int r = d / 2; r < ATF_MAX_PAIRS; ++r) th.t[r] = 0.0;
-  const int64_t threads = N * (d / 16);
-  const int64_t blocks = (threads + 255) / 256;
-  if (blocks > 0x7FFFFFFF) return atf_fail(ATF_ERR_UNSUPPORTED, "atf_rope: N too large");
-  const int BH = B * H;
-  // enough blocks along y to fill the GPU when N is short, few enough to amortise sincos
-  int gy = 1;
-  while (gy < BH && blocks * gy < 148 * 8) gy *= 2;
-  if (gy > BH) gy = BH;
-  dim3 grid((unsigned)blocks, (unsigned)gy);
-  cudaStream_t s = (cudaStream_t)stream;
-  if (d == 64)
-    atf_rope_kernel<64><<<grid, 256, 0, s>>>((__nv_bfloat16*)X, BH, N, pos0, th);
-  else
-    atf_rope_kernel<128><<<grid, 256, 0, s>>>((__nv_bfloat16*)X, BH, N, pos0, th);
-  ATF_CUDA_CHECK(cudaGetLastError());
-  return ATF_OK;
+extern "C" atf_status atf_rope_f32(float* X, int B, int H, int64_t N, int d, const double* theta, int64_t pos0, void* stream) {
+  return rope("atf_rope_f32", X, B, H, N, d, theta, pos0, stream);
+}
+
+extern "C" atf_status atf_rope(void* X, int B, int H, int64_t N, int d, const double* theta, int64_t pos0, void* stream) {
+  return rope("atf_rope", (__nv_bfloat16*)X, B, H, N, d, theta, pos0, stream);
 }
