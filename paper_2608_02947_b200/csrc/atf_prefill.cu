@@ -2,8 +2,9 @@
 // tensor cores.  This file holds the host side (validation, workspace, tensor maps, entry points)
 // and the layout pre-pass; the kernel is in atf_prefill_pipe.cu.
 //
-// Data layout.  A pre-pass copies Q and K into a pair-interleaved column order, lowest
-// frequency first: column 2p holds dim (h-1-p), column 2p+1 holds dim (d-1-p), h = d/2.  A
+// Data layout.  A pre-pass copies K into a pair-interleaved column order, lowest frequency first:
+// column 2p holds dim (h-1-p), column 2p+1 holds dim (d-1-p), h = d/2; the kernel puts its rows of
+// Q into the same order as it reads them (a row of Q is read by one CTA, one of K by many).  A
 // query-key dot product does not change under a common column permutation, and in this order
 // the pairs that are live at a distance (a contiguous low-frequency slice, Sec. 3.3) are a
 // PREFIX of the columns, so "advance the start of the pair loop" becomes "contract over the
@@ -19,37 +20,48 @@ namespace {
 
 constexpr int T = 128;  // query rows per tile and key columns per tile
 
-__global__ void __launch_bounds__(256)
-atf_repack_kernel(const __nv_bfloat16* __restrict__ X, __nv_bfloat16* __restrict__ Y, int64_t rows, int D,
-                  int64_t n_per_head, int64_t src_head_rows, __nv_bfloat16* __restrict__ Kg, int64_t kg_tiles,
-                  int64_t kg_first_row) {
-  // one thread writes 8 consecutive output columns (4 pairs) of one row; the source holds
-  // src_head_rows rows per head of which the first n_per_head are copied, the result is dense.
-  // With Kg the same 16 bytes also go into the tiled group-major K cache (kg_tiles tiles per head), for
-  // the rows from kg_first_row on: a group of that cache is two such 16-byte pieces of a key.
-  const int H = D / 2;
-  const int per_row = D / 8;
-  const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// The pre-pass, one launch: band schedule, and K in the column order above.  One thread moves eight pairs of a row: 16
+// bytes of each half row become 32 bytes of output, so that the pass is bound by memory (8 heads x 8192 rows of 128 into
+// the copy and the cache: 11.7 us from cold caches, 50 MB).  The source holds src_head_rows rows per head of which the
+// first n_per_head are copied, the result is dense.
+// With Kg the same eight pairs, a group of the tiled group-major K cache (kg_tiles tiles per head), also go there for the
+// rows from kg_first_row on.
+__global__ void __launch_bounds__(ATF_PREP_THREADS)
+atf_prefill_prep_kernel(const __grid_constant__ AtfTable table, int mode, int ndt, int sched_blocks, uint32_t* __restrict__ sched,
+                        const __nv_bfloat16* __restrict__ X, __nv_bfloat16* __restrict__ Y, int64_t rows, int D,
+                        int64_t n_per_head, int64_t src_head_rows, __nv_bfloat16* __restrict__ Kg, int64_t kg_tiles,
+                        int64_t kg_first_row) {
+  grid_dependency_launch();
+  const int H = D / 2, per_row = D / 16;
+  if ((int)blockIdx.x < sched_blocks) return atf_write_schedule(table, mode, H, ndt, sched);
+  const int64_t gid = (int64_t)(blockIdx.x - sched_blocks) * ATF_PREP_THREADS + threadIdx.x;
   if (gid >= rows * per_row) return;
   const int64_t row = gid / per_row;
-  const int t = (int)(gid % per_row);
+  const int c = (int)(gid % per_row);           // dims 8c .. 8c + 7 of each half, pairs 8j .. 8j + 7 in falling order
+  const int j = per_row - 1 - c;
   const int64_t head = row / n_per_head;
   const int64_t m = row - head * n_per_head;  // position of the row in its head
-  const __nv_bfloat16* src = X + (head * src_head_rows + m) * D;
-  __align__(16) __nv_bfloat16 out[8];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int p = 4 * t + i;
-    out[2 * i] = src[H - 1 - p];
-    out[2 * i + 1] = src[D - 1 - p];
-  }
-  *reinterpret_cast<uint4*>(Y + row * D + 8 * t) = *reinterpret_cast<const uint4*>(out);
+  const __nv_bfloat16* src = X + (head * src_head_rows + m) * D + 8 * c;
+  const uint4 lo = *reinterpret_cast<const uint4*>(src), hi = *reinterpret_cast<const uint4*>(src + H);
+  uint4 a, b;
+  a.x = __byte_perm(lo.w, hi.w, 0x7632);
+  a.y = __byte_perm(lo.w, hi.w, 0x5410);
+  a.z = __byte_perm(lo.z, hi.z, 0x7632);
+  a.w = __byte_perm(lo.z, hi.z, 0x5410);
+  b.x = __byte_perm(lo.y, hi.y, 0x7632);
+  b.y = __byte_perm(lo.y, hi.y, 0x5410);
+  b.z = __byte_perm(lo.x, hi.x, 0x7632);
+  b.w = __byte_perm(lo.x, hi.x, 0x5410);
+  uint4* dst = reinterpret_cast<uint4*>(Y + row * D + 16 * j);
+  dst[0] = a;
+  dst[1] = b;
   if (Kg && m >= kg_first_row) {
     const int64_t KT = 8192 / D;  // keys per 16 KiB tile
     const int64_t tile = m / KT, kin = m % KT;
-    const int j = t >> 1, half = (t & 1) ^ (int)((kin >> 2) & 1);
-    *reinterpret_cast<uint4*>(Kg + (((head * kg_tiles + tile) * (D / 16) + j) * KT + kin) * 16 + half * 8) =
-        *reinterpret_cast<const uint4*>(out);
+    const int swap = (int)((kin >> 2) & 1);  // keys with bit 2 set store their two 16-byte halves swapped
+    uint4* g = reinterpret_cast<uint4*>(Kg + (((head * kg_tiles + tile) * (D / 16) + j) * KT + kin) * 16);
+    g[swap] = a;
+    g[swap ^ 1] = b;
   }
 }
 
@@ -108,32 +120,31 @@ atf_status atf_prefill_impl(const void* Q, const void* K, const void* V, void* O
 
   char* base = (char*)ws.ptr;
   uint32_t* sched = (uint32_t*)(base + ATF_WS_HEADER);
-  __nv_bfloat16* Qp = (__nv_bfloat16*)(base + ATF_WS_HEADER + sched_bytes(N));
-  __nv_bfloat16* Kp = (__nv_bfloat16*)(base + ATF_WS_HEADER + sched_bytes(N) + repack_bytes(B, Hq, Nq, d));
+  __nv_bfloat16* Kp = (__nv_bfloat16*)(base + ATF_WS_HEADER + sched_bytes(N));
   cudaStream_t s = (cudaStream_t)stream;
 
   {
     const int64_t rows_q = (int64_t)B * Hq * Nq, rows_k = (int64_t)B * Hkv * N;
-    const int64_t bq = (rows_q * (d / 8) + 255) / 256, bk = (rows_k * (d / 8) + 255) / 256;
-    if (bq > 0x7FFFFFFF) return atf_fail(ATF_ERR_UNSUPPORTED, "atf_prefill: problem too large for the repack grid");
+    if ((rows_q * (d / 8) + 255) / 256 > 0x7FFFFFFF) return atf_fail(ATF_ERR_UNSUPPORTED, "atf_prefill: problem too large for the repack grid");
+    const int sb = atf_sched_blocks(N);
+    const int64_t blocks = sb + (rows_k * (d / 16) + ATF_PREP_THREADS - 1) / ATF_PREP_THREADS;
+    if (blocks > 0x7FFFFFFF) return atf_fail(ATF_ERR_UNSUPPORTED, "atf_prefill: problem too large for the repack grid");
     __nv_bfloat16* Kg = opts ? (__nv_bfloat16*)opts->kcache_groups : nullptr;
     const int64_t kt = 8192 / d;
     const int64_t kg_tiles = Kg ? (opts->kcache_capacity + kt - 1) / kt : 0;
-    atf_repack_kernel<<<(unsigned)bq, 256, 0, s>>>((const __nv_bfloat16*)Q, Qp, rows_q, d, Nq, Nq, nullptr, 0, 0);
-    atf_repack_kernel<<<(unsigned)bk, 256, 0, s>>>((const __nv_bfloat16*)K, Kp, rows_k, d, N, kv_head_rows, Kg, kg_tiles,
-                                                   N - Nq);
+    atf_prefill_prep_kernel<<<(unsigned)blocks, ATF_PREP_THREADS, 0, s>>>(
+        t, mode, (int)((N + T - 1) / T), sb, sched, (const __nv_bfloat16*)K, Kp, rows_k, d, N, kv_head_rows, Kg, kg_tiles, N - Nq);
     ATF_CUDA_CHECK(cudaGetLastError());
   }
 
-  CUtensorMap tq, tk, tv;
-  if ((st = atf_make_tile_map(&tq, Qp, (int64_t)B * Hq, Nq, d, Nq, T)) != ATF_OK) return st;
+  CUtensorMap tk, tv;
   if ((st = atf_make_tile_map(&tk, Kp, (int64_t)B * Hkv, N, d, N, T)) != ATF_OK) return st;
   if ((st = atf_make_tile_map(&tv, V, (int64_t)B * Hkv, N, d, kv_head_rows, T)) != ATF_OK) return st;
 
   AtfPipeParams P;
   P.sched = sched;
-  P.Qp = Qp;
-  P.Qp_lo = nullptr;
+  P.Q = (const __nv_bfloat16*)Q;
+  P.Qhi = P.Qlo = nullptr;
   P.O = (__nv_bfloat16*)O;
   P.LSE = LSE;
   P.kept = opts ? (unsigned long long*)opts->kept_terms : nullptr;
@@ -142,7 +153,7 @@ atf_status atf_prefill_impl(const void* Q, const void* K, const void* V, void* O
   P.Hkv = Hkv;
   P.N = (int)N;
   P.Nq = (int)Nq;
-  return atf_launch_prefill_pipe(tq, tk, tv, P, t, B, d, mode, P.kept != nullptr, s);
+  return atf_launch_prefill_pipe(tk, tv, P, t, B, d, mode, P.kept != nullptr, s);
 }
 
 extern "C" atf_status atf_prefill_chunk_ex(const void* Q, const void* K, const void* V, void* O, float* LSE, int B,

@@ -4,13 +4,20 @@
 // With a single query tile the 512 tensor-memory columns hold two S buffers, two P buffers and O, so
 // the chain "softmax -> O += P V -> next S -> softmax" is cut: S(t + 1) = Q K(t + 1)^T is computed
 // while the softmax groups work on S(t), and O += P(t) V runs whenever P(t) is stored.  Warp roles:
-//   warp 0      TMA producer: Q (again per pass, see below), K (live 64-column blocks) and V
-//               tiles into three-stage rings of 128-byte-swizzled shared memory;
+//   warp 0      TMA producer: K (live 64-column blocks) and V tiles into three-stage rings of
+//               128-byte-swizzled shared memory;
 //   warp 1      issuer of S(t) = Q K(t)^T over the live depth (one thread, tcgen05.mma SS form);
 //   warp 2      issuer of O += P(t) V(t), half a tile at a time (one thread, TS form: P is read from
 //               tensor memory, V through the MN-major descriptor);
 //   warps 4-7   softmax group 0: keys 0..63 of every tile, one query row per thread;
 //   warps 8-11  softmax group 1: keys 64..127 of the same rows.
+// The softmax warps also bring Q in (half a row each, again per pass, see below): they read the caller's rows and
+// store them to shared memory in the column order of atf_prefill.cu.  A row of Q is read by one CTA only, so a pre-pass
+// that reorders it would move it twice more (8192 rows of 24 heads: 22 us of 700).  The split-precision mode keeps such
+// a pre-pass and loads Q by TMA: splitting fp32 rows here took longer (10001 rows: 1.21 against 1.19 ms).  Exact mode
+// holds a second, whole copy for the per-cell finish, where a pair fetched from global memory cost an L2 round trip
+// (8192 rows: 733 us against 685); at d = 128 that leaves two K stages, which long rows feel (131072 rows: + 1 %).
+// The launch overlaps the end of the pre-pass (programmatic dependent launch): everything up to Q needs nothing of it.
 // The two threads of a row never meet in the common step: exponentials are taken against the
 // row's reference maximum from the diagonal tile (any reference gives the same softmax as long
 // as nothing overflows: P is bf16, O and the row sums are fp32), each thread keeps its own
@@ -53,18 +60,21 @@ static_assert(128 * 56 + 256 * 224 <= PP_THREADS * 168, "setmaxnreg budget excee
 
 // SPLIT (the split-precision mode, atf_prefill_split.cu): Q and K come as bf16 hi and lo parts; the CTA holds both
 // Q parts, a K stage is a hi tile followed by a lo tile, and the rings shrink to two K stages and one V stage.
-template <int D, bool SPLIT>
+// QCOPY (exact mode, bf16 inputs): a second copy of Q that stays whole, for the per-cell finish; at d = 128 it takes the
+// place of the third K stage.
+template <int D, bool SPLIT, bool QCOPY>
 struct PipeSmem {
   static constexpr int NB = D / 64;
   static constexpr int TILE = NB * BLK_BYTES;
   static constexpr int QN = SPLIT ? 2 : 1;       // operand parts: hi, lo
-  static constexpr int KS = SPLIT ? 2 : 3;       // ring depths
+  static constexpr int KS = SPLIT || (QCOPY && D == 128) ? 2 : 3;  // ring depths
   static constexpr int VS = SPLIT ? 1 : 3;
   static constexpr int KSTAGE = QN * TILE;
   static constexpr int Q_OFF = 0;                // hi part, then lo part
   static constexpr int K_OFF = QN * TILE;
   static constexpr int V_OFF = K_OFF + KS * KSTAGE;
-  static constexpr int BAR_OFF = V_OFF + VS * TILE;
+  static constexpr int QC_OFF = V_OFF + VS * TILE;
+  static constexpr int BAR_OFF = QC_OFF + (QCOPY ? TILE : 0);
   static constexpr int X_OFF = BAR_OFF + 256;  // exchange area of the two softmax groups: [2][128] floats
   static constexpr int TOTAL = X_OFF + 1024;
   static constexpr int DYN_BYTES = TOTAL + 1024;  // slack for 1024-byte alignment
@@ -126,7 +136,7 @@ __device__ __forceinline__ void mma_16816(float* c, uint32_t a0, uint32_t a1, ui
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-// Band schedule (Sec. 3.3: the active pairs of a tile are known statically).  What a step needs depends only on
+// Band schedule (Sec. 3.3: the active pairs of a tile are known statically; written by atf_write_schedule, atf_prefill_pipe.cuh).  What a step needs depends only on
 // the tile distance dt and on which 32 rows x 64 keys of the tile a softmax warp owns (quarter wq of the rows,
 // half h of the keys); it is the same for every CTA of a launch.  A pre-kernel writes one word per (dt, wq, h):
 //   p_all  [0:7)   pairs live in every cell of the warp's block,      p_any [7:14)  pairs live in some cell of it,
@@ -142,39 +152,6 @@ struct PipeWord {
       : p_all(e & 127), p_any((e >> 7) & 127), p_mid((e >> 14) & 127), natoms((e >> 21) & 15), nkb(((e >> 25) & 3) + 1),
         plain((e >> 27) & 1) {}
 };
-
-template <int MODE>
-__global__ void __launch_bounds__(128)
-atf_pipe_sched_kernel(const __grid_constant__ AtfTable table, int H, int ndt, uint32_t* __restrict__ out) {
-  // one thread per word: 16 tile distances x 8 (quarter, half) blocks per CTA, the table in shared memory
-  __shared__ int w[ATF_MAX_PAIRS];
-  if (threadIdx.x < H) w[threadIdx.x] = table.w[threadIdx.x];
-  __syncthreads();
-  const int dt = blockIdx.x * 16 + (threadIdx.x >> 3);
-  if (dt >= ndt) return;
-  const int wq = (threadIdx.x >> 1) & 3, h = threadIdx.x & 1;
-  const int Wmax = w[H - 1];
-  auto reaching = [&](int z) {  // pairs (from the low-frequency end) whose window reaches distance z
-    int lo = 0, hi = H;         // first r with w[r] >= z, w non-decreasing
-    while (lo < hi) {
-      const int mid = (lo + hi) >> 1;
-      if (w[mid] < z) lo = mid + 1; else hi = mid;
-    }
-    return H - lo;
-  };
-  const int tile_any = reaching(dt == 0 ? 0 : dt * T - (T - 1));  // live somewhere in the tile
-  const int mid0 = reaching(dt == 0 ? 15 : dt * T - 48);           // what the nearest quarter keeps in the MMA
-  const int natoms = MODE == ATF_MODE_EXACT ? (mid0 + 7) / 8 : (dt == 0 ? H / 8 : (tile_any + 7) / 8);
-  const int cols = MODE == ATF_MODE_EXACT ? 2 * tile_any : 16 * natoms;  // exact mode also reads the pairs it adds per cell
-  const int nkb = max(1, (cols + 63) / 64);
-  const int zmax = dt * T + 32 * wq + 31 - 64 * h, zmin = dt * T + 32 * wq - 64 * h - 63;
-  const int p_all = reaching(max(0, zmax)), p_any = reaching(max(0, zmin));
-  const int p_mid = reaching(dt == 0 ? 16 * wq + 15 : dt * T + 32 * wq - 48);
-  bool plain = dt > 0 && natoms > 0;
-  if (MODE == ATF_MODE_EXACT) plain = plain && zmax <= Wmax && min(p_all, p_mid) >= max(p_any, p_mid);
-  out[8 * dt + 2 * wq + h] = (uint32_t)p_all | ((uint32_t)p_any << 7) | ((uint32_t)p_mid << 14) | ((uint32_t)natoms << 21) |
-                             ((uint32_t)(nkb - 1) << 25) | ((uint32_t)plain << 27);
-}
 
 __device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
   if (mbar_try_wait(bar, parity)) return true;
@@ -197,7 +174,8 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                         const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmKlo,
                         const __grid_constant__ CUtensorMap tmV, const __grid_constant__ AtfPipeParams P,
                         const __grid_constant__ AtfTable table) {
-  using SM = PipeSmem<D, SPLIT>;
+  constexpr bool QCOPY = MODE == ATF_MODE_EXACT && !SPLIT;
+  using SM = PipeSmem<D, SPLIT, QCOPY>;
   constexpr int KS = SM::KS, VS = SM::VS;
   constexpr int POLY = SPLIT ? 0 : ATF_PIPE_POLY_OF_4;
   constexpr int H = D / 2;
@@ -231,7 +209,7 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   if (tid == 0) {
     s_abort = 0;
     s_redo = 0;
-    mbar_init(bar(B_QFULL), 1);
+    mbar_init(bar(B_QFULL), SPLIT ? 1 : 8);
     mbar_init(bar(B_OFULL), 1);
     mbar_init(bar(B_XCH), 8);
     mbar_init(bar(B_QZ), 4);
@@ -251,9 +229,9 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     }
     mbar_fence_init();
     fence_proxy_async_smem();
-    tma_prefetch_desc(&tmQ);
     tma_prefetch_desc(&tmK);
     if (SPLIT) {
+      tma_prefetch_desc(&tmQ);
       tma_prefetch_desc(&tmQlo);
       tma_prefetch_desc(&tmKlo);
     }
@@ -284,14 +262,17 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   if (warp == 0) {
     // =============================== TMA producer ===============================
     asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+    grid_dependency_wait();
     for (int pass = 0; pass < 2; ++pass) {
       const int g0 = pass * nt;
       if (lane == 0) {
-        mbar_expect_tx(bar(B_QFULL), SM::QN * SM::TILE);
-        for (int kb = 0; kb < NB; ++kb) {
-          // rows before n0 do not exist in Q: the (possibly negative) coordinate reads zero fill there
-          tma_load_3d(sQ + kb * BLK_BYTES, &tmQ, bar(B_QFULL), kb * 64, it * T - n0, bhq);
-          if (SPLIT) tma_load_3d(sQ + SM::TILE + kb * BLK_BYTES, &tmQlo, bar(B_QFULL), kb * 64, it * T - n0, bhq);
+        if (SPLIT) {
+          mbar_expect_tx(bar(B_QFULL), SM::QN * SM::TILE);
+          for (int kb = 0; kb < NB; ++kb) {
+            // rows before n0 do not exist in Q: the (possibly negative) coordinate reads zero fill there
+            tma_load_3d(sQ + kb * BLK_BYTES, &tmQ, bar(B_QFULL), kb * 64, it * T - n0, bhq);
+            tma_load_3d(sQ + SM::TILE + kb * BLK_BYTES, &tmQlo, bar(B_QFULL), kb * 64, it * T - n0, bhq);
+          }
         }
         auto load_k = [&](int t) {
           const int g = g0 + t, ks = g % KS;
@@ -328,6 +309,7 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   } else if (warp == 1) {
     // =============================== issuer of S = Q K^T ===============================
     asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+    grid_dependency_wait();
     for (int pass = 0; pass < 2; ++pass) {
       const int g0 = pass * nt;
       if (lane == 0) {
@@ -405,8 +387,9 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     const int64_t qrow = (int64_t)bhq * P.Nq + (row_ok ? n - n0 : 0);
     const uint32_t lane_off = (uint32_t)(wq * 32) << 16;
     const uint32_t tO = tmem_base + 2 * T + lane_off;
-    const __nv_bfloat16* qsrc = P.Qp + qrow * D;
-    const __nv_bfloat16* qsrc_lo = SPLIT ? P.Qp_lo + qrow * D : nullptr;
+    // split mode: the hi and lo parts of this row, pairs in column order
+    const uint32_t* qsrc = SPLIT ? reinterpret_cast<const uint32_t*>(P.Qhi + qrow * D) : nullptr;
+    const uint32_t* qsrc_lo = SPLIT ? reinterpret_cast<const uint32_t*>(P.Qlo + qrow * D) : nullptr;
     float m_used = -INFINITY, l_run = 0.f;
     unsigned long long cnt = 0;
     uint32_t xphase = 0;
@@ -419,9 +402,26 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       ++xphase;
       return r;
     };
+    // This group's half of the pairs of the row, p = h H/2 + i: dims H-1-p and D-1-p, which are QW consecutive elements of
+    // each half row in falling order.  Rows that do not exist (before n0, from N on) are zero.
+    constexpr int QW = H / 2;
+    auto load_q = [&](uint32_t (&w)[QW]) {
+      const __nv_bfloat16* q = P.Q + qrow * D + (H - QW - h * QW);
+      uint32_t x[QW / 2], y[QW / 2];
+#pragma unroll
+      for (int i = 0; i < QW / 2; i += 4) {
+        *reinterpret_cast<uint4*>(x + i) = row_ok ? __ldg(reinterpret_cast<const uint4*>(q + 2 * i)) : make_uint4(0u, 0u, 0u, 0u);
+        *reinterpret_cast<uint4*>(y + i) = row_ok ? __ldg(reinterpret_cast<const uint4*>(q + H + 2 * i)) : make_uint4(0u, 0u, 0u, 0u);
+      }
+#pragma unroll
+      for (int i = 0; i < QW; ++i) w[i] = __byte_perm(x[(QW - 1 - i) >> 1], y[(QW - 1 - i) >> 1], (i & 1) ? 0x5410 : 0x7632);
+    };
     for (int pass = 0; pass < 2; ++pass) {
       const int g0 = pass * nt;
       const bool safe = pass == 1;
+      uint32_t qw[QW];
+      if constexpr (!SPLIT) load_q(qw);
+      if (pass == 0) grid_dependency_wait();
       m_used = -INFINITY;
       l_run = 0.f;
       cnt = 0;
@@ -445,9 +445,31 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       const uint32_t* sched = P.sched + 2 * wq + h;
       uint32_t e_cur = __ldg(sched);  // schedule word of the step at hand; the next one is fetched a step ahead
       int p_mid = PipeWord(e_cur).p_mid;
-      if (MODE == ATF_MODE_EXACT) {
-        if (ok && !wait_or_abort(bar(B_QFULL), pass & 1, abortp)) { ok = false; fail_site = 30; }
-        if (ok) zero_q_down_to(p_mid);
+      if constexpr (SPLIT) {
+        if (MODE == ATF_MODE_EXACT) {
+          if (ok && !wait_or_abort(bar(B_QFULL), pass & 1, abortp)) { ok = false; fail_site = 30; }
+          if (ok) zero_q_down_to(p_mid);
+        }
+      } else {
+        // ---- Q: this group's half of the pairs of the row, p = h H/2 + i.  Exact mode: what the first MMA does not take
+        //      is zero, and the copy stays whole. ----
+        const int p_keep = MODE == ATF_MODE_EXACT ? p_mid : H;
+#pragma unroll
+        for (int c = 0; c < QW / 4; ++c) {
+          const int p = h * QW + 4 * c;
+          const uint32_t off = (p >> 5) * BLK_BYTES + sw128_offset(row, (p & 31) >> 2);
+          *reinterpret_cast<uint4*>(smem_gen + SM::Q_OFF + off) =
+              make_uint4(p < p_keep ? qw[4 * c] : 0u, p + 1 < p_keep ? qw[4 * c + 1] : 0u,
+                         p + 2 < p_keep ? qw[4 * c + 2] : 0u, p + 3 < p_keep ? qw[4 * c + 3] : 0u);
+          if (QCOPY) *reinterpret_cast<uint4*>(smem_gen + SM::QC_OFF + off) = make_uint4(qw[4 * c], qw[4 * c + 1], qw[4 * c + 2], qw[4 * c + 3]);
+        }
+        zeroed_from = p_keep;
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) {
+          mbar_arrive(bar(B_QFULL));
+          if (MODE == ATF_MODE_EXACT && h == 0) mbar_arrive(bar(B_QZ));
+        }
       }
       int t = 0;
       while (t < nt && ok) {
@@ -494,7 +516,6 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         const int dt = t;
         const int zrow = dt * T + row;             // distance from this row to column 0 of the key tile
         const int zmax_w = dt * T + 32 * wq + 31 - 64 * h;  // over the warp's 32 x 64 cells
-        const int zmin_w = dt * T + 32 * wq - 64 * h - 63;
         const PipeWord E(e_cur);
         const uint32_t e_next = t + 1 < nt ? __ldg(sched + 8 * (t + 1)) : 0u;
         const int p_all = E.p_all, p_any = E.p_any, natoms = E.natoms;
@@ -516,8 +537,20 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
           //      accumulator-fragment order. ----
           const int p_lo = min(p_all, p_mid), p_hi = max(p_any, p_mid);
           if (p_lo < p_hi && zmax_w >= 0) {
-            uint32_t q_next = *reinterpret_cast<const uint32_t*>(qsrc + 2 * p_lo), ql_next = 0u;
-            if (SPLIT) ql_next = *reinterpret_cast<const uint32_t*>(qsrc_lo + 2 * p_lo);
+            uint32_t q_next = 0u, ql_next = 0u;
+            const uint32_t qrow0 = smem_base + SM::QC_OFF + (32 * wq + (lane >> 2)) * 128;
+            uint32_t qr_next[4];  // QCOPY: the pair of rows lane / 4 + 8 j, fetched a pair ahead
+            auto fetch_q = [&](int p) {
+              if (QCOPY) {
+                const uint32_t a = qrow0 + (p >> 5) * BLK_BYTES + ((((p & 31) >> 2) ^ (lane >> 2)) << 4) + (p & 3) * 4;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) asm volatile("ld.shared.b32 %0, [%1];" : "=r"(qr_next[j]) : "r"(a + j * 1024));
+              } else {
+                q_next = qsrc[p];
+                ql_next = qsrc_lo[p];
+              }
+            };
+            fetch_q(p_lo);
             if (!wait_or_abort(bar(B_KFULL + ks), (g / KS) & 1, abortp)) { ok = false; fail_site = 32; break; }
             float f[2][32];  // rows 16 hf + {lane / 4, lane / 4 + 8}, keys 64h + 8 cb + 2 (lane % 4) + {0, 1}
             if (s_valid) {
@@ -537,17 +570,14 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             for (int p = p_lo; p < p_hi; ++p) {
               const bool subtract = p < p_mid;
               const uint32_t flip = subtract ? 0x80008000u : 0u;
-              const uint32_t qq = q_next ^ flip, ql = ql_next ^ flip;
-              const int pn = min(p + 1, p_hi - 1);
-              q_next = *reinterpret_cast<const uint32_t*>(qsrc + 2 * pn);
-              if (SPLIT) ql_next = *reinterpret_cast<const uint32_t*>(qsrc_lo + 2 * pn);
-              const int wp = sW[H - 1 - p];
               uint32_t qr[4], qrl[SPLIT ? 4 : 1];  // the pair of rows g8 + 8 j
 #pragma unroll
               for (int j = 0; j < 4; ++j) {
-                qr[j] = __shfl_sync(0xffffffffu, qq, g8 + 8 * j);
-                if (SPLIT) qrl[j] = __shfl_sync(0xffffffffu, ql, g8 + 8 * j);
+                qr[j] = QCOPY ? qr_next[j] ^ flip : __shfl_sync(0xffffffffu, q_next, g8 + 8 * j) ^ flip;
+                if (SPLIT) qrl[j] = __shfl_sync(0xffffffffu, ql_next, g8 + 8 * j) ^ flip;
               }
+              if (p + 1 < p_hi) fetch_q(p + 1);
+              const int wp = sW[H - 1 - p];
               // row g8 + 8 j takes the key of slot t4 (t4 + 4) of block cb inside the window iff 8 (cb - j) >= u (u - 4)
               const int u = zw_lo + g8 - t4 - 64 * h - wp;
               const uint32_t kp = krow + ((2 * p) >> 6) * BLK_BYTES + (((((2 * p) & 63) >> 3) ^ g8) << 4) + ((2 * p) & 7) * 2;
@@ -728,17 +758,22 @@ atf_status launch_pipe(const CUtensorMap& tq, const CUtensorMap& tql, const CUte
                        cudaStream_t s) {
   const int ntq = (P.N + T - 1) / T;
   const int it0 = (P.N - P.Nq) / T;  // first tile with a query row
-  dim3 grid(ntq - it0, P.Hq, B);
-  if (mode == ATF_MODE_EXACT)
-    atf_pipe_sched_kernel<ATF_MODE_EXACT><<<(ntq + 15) / 16, 128, 0, s>>>(t, D / 2, ntq, P.sched);
-  else
-    atf_pipe_sched_kernel<ATF_MODE_COARSE><<<(ntq + 15) / 16, 128, 0, s>>>(t, D / 2, ntq, P.sched);
-  const int smem = PipeSmem<D, SPLIT>::DYN_BYTES;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(ntq - it0, P.Hq, B);
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  cfg.blockDim = dim3(PP_THREADS);
 #define ATF_PP_LAUNCH(MODE_, COUNT_)                                                                   \
   do {                                                                                                 \
     auto kern = atf_prefill_pipe_kernel<D, MODE_, COUNT_, SPLIT>;                                      \
+    const int smem = PipeSmem<D, SPLIT, MODE_ == ATF_MODE_EXACT && !SPLIT>::DYN_BYTES;                 \
     ATF_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));     \
-    kern<<<grid, PP_THREADS, smem, s>>>(tq, tql, tk, tkl, tv, P, t);                                   \
+    cfg.dynamicSmemBytes = smem;                                                                       \
+    ATF_CUDA_CHECK(cudaLaunchKernelEx(&cfg, kern, tq, tql, tk, tkl, tv, P, t));                        \
   } while (0)
   if (mode == ATF_MODE_EXACT) {
     if (count) ATF_PP_LAUNCH(ATF_MODE_EXACT, true); else ATF_PP_LAUNCH(ATF_MODE_EXACT, false);
@@ -752,11 +787,10 @@ atf_status launch_pipe(const CUtensorMap& tq, const CUtensorMap& tql, const CUte
 
 }  // namespace
 
-atf_status atf_launch_prefill_pipe(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
-                                   const AtfPipeParams& P, const AtfTable& t, int B, int d, int mode, bool count,
-                                   cudaStream_t s) {
-  return d == 64 ? launch_pipe<64, false>(tq, tq, tk, tk, tv, P, t, B, mode, count, s)
-                 : launch_pipe<128, false>(tq, tq, tk, tk, tv, P, t, B, mode, count, s);
+atf_status atf_launch_prefill_pipe(const CUtensorMap& tk, const CUtensorMap& tv, const AtfPipeParams& P,
+                                   const AtfTable& t, int B, int d, int mode, bool count, cudaStream_t s) {
+  return d == 64 ? launch_pipe<64, false>(tk, tk, tk, tk, tv, P, t, B, mode, count, s)
+                 : launch_pipe<128, false>(tk, tk, tk, tk, tv, P, t, B, mode, count, s);
 }
 
 atf_status atf_launch_prefill_pipe_split(const CUtensorMap& tqh, const CUtensorMap& tql, const CUtensorMap& tkh,

@@ -23,30 +23,42 @@ namespace {
 
 constexpr int T = 128;
 
-// hi = bf16(x), lo = bf16(x - hi), written in the pair-interleaved column order: column 2p holds
-// dim (h-1-p), column 2p+1 holds dim (d-1-p).  One thread writes 8 consecutive output columns.
-__global__ void __launch_bounds__(256)
-atf_split_repack_kernel(const float* __restrict__ X, __nv_bfloat16* __restrict__ Yhi, __nv_bfloat16* __restrict__ Ylo,
-                        int64_t rows, int D) {
-  const int H = D / 2;
-  const int per_row = D / 8;
-  const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (gid >= rows * per_row) return;
-  const int64_t row = gid / per_row;
-  const int t = (int)(gid % per_row);
-  const float* src = X + row * D;
-  __align__(16) __nv_bfloat16 hi[8], lo[8];
+// The pre-pass, one launch: band schedule, then hi = bf16(x), lo = bf16(x - hi) of Q and of K in the pair-interleaved
+// column order.  One thread moves eight pairs of a row; memory bounds it (10001 rows of 24 + 8 heads of 128: 49 us, 327 MB).
+__global__ void __launch_bounds__(ATF_PREP_THREADS)
+atf_split_prep_kernel(const __grid_constant__ AtfTable table, int mode, int ndt, int sched_blocks, uint32_t* __restrict__ sched,
+                      const float* __restrict__ Q, const float* __restrict__ K, __nv_bfloat16* __restrict__ Qhi,
+                      __nv_bfloat16* __restrict__ Qlo, __nv_bfloat16* __restrict__ Khi, __nv_bfloat16* __restrict__ Klo,
+                      int64_t rows_q, int64_t rows_k, int D) {
+  grid_dependency_launch();
+  const int H = D / 2, per_row = D / 16;
+  if ((int)blockIdx.x < sched_blocks) return atf_write_schedule(table, mode, H, ndt, sched);
+  const int64_t gid = (int64_t)(blockIdx.x - sched_blocks) * ATF_PREP_THREADS + threadIdx.x;
+  int64_t row = gid / per_row;
+  const int c = (int)(gid % per_row);           // dims 8c .. 8c + 7 of each half, pairs 8j .. 8j + 7 in falling order
+  if (row >= rows_q + rows_k) return;
+  const bool is_k = row >= rows_q;
+  if (is_k) row -= rows_q;
+  const float* src = (is_k ? K : Q) + row * D + 8 * c;
+  float x[8], y[8];
+  *reinterpret_cast<float4*>(x) = *reinterpret_cast<const float4*>(src);
+  *reinterpret_cast<float4*>(x + 4) = *reinterpret_cast<const float4*>(src + 4);
+  *reinterpret_cast<float4*>(y) = *reinterpret_cast<const float4*>(src + H);
+  *reinterpret_cast<float4*>(y + 4) = *reinterpret_cast<const float4*>(src + H + 4);
+  uint32_t hi[8], lo[8];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int p = 4 * t + i;
-    const float a = src[H - 1 - p], b = src[D - 1 - p];
-    hi[2 * i] = __float2bfloat16_rn(a);
-    hi[2 * i + 1] = __float2bfloat16_rn(b);
-    lo[2 * i] = __float2bfloat16_rn(a - __bfloat162float(hi[2 * i]));
-    lo[2 * i + 1] = __float2bfloat16_rn(b - __bfloat162float(hi[2 * i + 1]));
+  for (int i = 0; i < 8; ++i) {
+    const float a = x[7 - i], b = y[7 - i];
+    hi[i] = pack_bf16x2(a, b);
+    lo[i] = pack_bf16x2(a - bf16lo_to_f32(hi[i]), b - bf16hi_to_f32(hi[i]));
   }
-  *reinterpret_cast<uint4*>(Yhi + row * D + 8 * t) = *reinterpret_cast<const uint4*>(hi);
-  *reinterpret_cast<uint4*>(Ylo + row * D + 8 * t) = *reinterpret_cast<const uint4*>(lo);
+  const int64_t off = row * D + 16 * (per_row - 1 - c);
+  uint4* dh = reinterpret_cast<uint4*>((is_k ? Khi : Qhi) + off);
+  uint4* dl = reinterpret_cast<uint4*>((is_k ? Klo : Qlo) + off);
+  dh[0] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+  dh[1] = make_uint4(hi[4], hi[5], hi[6], hi[7]);
+  dl[0] = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+  dl[1] = make_uint4(lo[4], lo[5], lo[6], lo[7]);
 }
 
 size_t part_bytes(int B, int H, int64_t N, int d) {
@@ -103,10 +115,13 @@ extern "C" atf_status atf_prefill_split_chunk(const float* Q, const float* K, co
   cudaStream_t s = (cudaStream_t)stream;
   {
     const int64_t rows_q = (int64_t)B * Hq * Nq, rows_k = (int64_t)B * Hkv * N;
-    const int64_t bq = (rows_q * (d / 8) + 255) / 256, bk = (rows_k * (d / 8) + 255) / 256;
-    if (bq > 0x7FFFFFFF) return atf_fail(ATF_ERR_UNSUPPORTED, "atf_prefill_split: problem too large for the repack grid");
-    atf_split_repack_kernel<<<(unsigned)bq, 256, 0, s>>>(Q, Qhi, Qlo, rows_q, d);
-    atf_split_repack_kernel<<<(unsigned)bk, 256, 0, s>>>(K, Khi, Klo, rows_k, d);
+    if ((rows_q * (d / 8) + 255) / 256 > 0x7FFFFFFF) return atf_fail(ATF_ERR_UNSUPPORTED, "atf_prefill_split: problem too large for the repack grid");
+    const int sb = atf_sched_blocks(N);
+    const int64_t blocks = sb + ((rows_q + rows_k) * (d / 16) + ATF_PREP_THREADS - 1) / ATF_PREP_THREADS;
+    if (blocks > 0x7FFFFFFF) return atf_fail(ATF_ERR_UNSUPPORTED, "atf_prefill_split: problem too large for the repack grid");
+    atf_split_prep_kernel<<<(unsigned)blocks, ATF_PREP_THREADS, 0, s>>>(t, mode, (int)((N + T - 1) / T), sb,
+                                                                        (uint32_t*)(base + ATF_WS_HEADER), Q, K, Qhi, Qlo, Khi,
+                                                                        Klo, rows_q, rows_k, d);
     ATF_CUDA_CHECK(cudaGetLastError());
   }
   CUtensorMap tqh, tql, tkh, tkl, tv;
@@ -118,8 +133,9 @@ extern "C" atf_status atf_prefill_split_chunk(const float* Q, const float* K, co
 
   AtfPipeParams P;
   P.sched = (uint32_t*)(base + ATF_WS_HEADER);
-  P.Qp = Qhi;
-  P.Qp_lo = Qlo;
+  P.Q = nullptr;
+  P.Qhi = Qhi;
+  P.Qlo = Qlo;
   P.O = (__nv_bfloat16*)O;
   P.LSE = LSE;
   P.kept = opts ? (unsigned long long*)opts->kept_terms : nullptr;
