@@ -1,7 +1,9 @@
 """ctypes binding of libatflash.so.  Argument marshalling only; every step runs in the library."""
 from __future__ import annotations
 
+import contextlib
 import ctypes as C
+import functools
 import math
 import os
 
@@ -142,16 +144,27 @@ def atf_window_table_family(base, d, N, scaling=None, profile="constant", k_hi=2
 
 
 def _stream(t):
-    return C.c_void_p(torch.cuda.current_stream(t.device).cuda_stream)
+    return C.c_void_p(_raw_stream(t))
+
+
+def _raw_stream(t):
+    """The stream handle that torch.cuda.current_stream(t.device).cuda_stream gives, without making the Stream object."""
+    return torch._C._cuda_getCurrentRawStream(t.device.index)
+
+
+_SAME_DEVICE = contextlib.nullcontext()
 
 
 def _one_device(*tensors):
     """All device tensors of a call must live on one GPU: the C side launches on the current device, and the
     binding makes that the tensors' device for the duration of the call."""
-    devs = {t.device for t in tensors if t is not None}
-    if len(devs) != 1:
-        raise AtfError(1, f"all tensors of a call must be on the same CUDA device (got {sorted(map(str, devs))})")
-    return torch.cuda.device(devs.pop())
+    dev = tensors[0].device
+    for t in tensors:
+        if t is not None and t.device != dev:
+            devs = {t.device for t in tensors if t is not None}
+            raise AtfError(1, f"all tensors of a call must be on the same CUDA device (got {sorted(map(str, devs))})")
+    # entering the device that is current already costs as much as the rest of a short call's checks
+    return _SAME_DEVICE if dev.index == torch.cuda.current_device() else torch.cuda.device(dev)
 
 
 def _dev_bf16(t, name):
@@ -181,6 +194,7 @@ def _table_ptr(table, d):
 _ws = None
 
 
+@functools.lru_cache(maxsize=256)
 def atf_workspace_bytes(op, B, Hq, Hkv, N, d):
     return int(lib().atf_workspace_bytes(op, B, Hq, Hkv, N, d))
 
@@ -246,8 +260,13 @@ def new_kcache_groups(B, Hkv, capacity, d, device):
     return torch.zeros((B, Hkv, (capacity + kt - 1) // kt, d // 16, kt, 16), dtype=torch.bfloat16, device=device)
 
 
+@functools.lru_cache(maxsize=16)
+def _tile_keys(d):
+    return int(lib().atf_kcache_tile_keys(d))
+
+
 def _check_kcache_groups(Kg, B, Hkv, N, d):
-    kt = int(lib().atf_kcache_tile_keys(d))
+    kt = _tile_keys(d)
     _dev_bf16(Kg, "kcache_groups")
     if Kg.dim() != 6 or Kg.shape[:2] != (B, Hkv) or Kg.shape[3:] != (d // 16, kt, 16) or Kg.shape[2] * kt < N:
         raise AtfError(1, f"kcache_groups must be [B,Hkv,tiles,d/16,{kt},16] with room for N keys")
@@ -467,9 +486,8 @@ def atf_decode(q, Kcache, Vcache, table=None, mode=ATF_MODE_EXACT, kept_terms=No
         o.rope_tables = rope_tables.buf.data_ptr()
         o.rope_tables_capacity = rope_tables.capacity
     with dev:
-        _check(lib().atf_decode_ex(C.c_void_p(q.data_ptr()), C.c_void_p(Kcache.data_ptr()), C.c_void_p(Vcache.data_ptr()),
-                                   C.c_void_p(O.data_ptr()), B, Hq, Hkv, L, d, tab,
-                                   C.byref(o) if o is not None else None, _stream(q)))
+        _check(lib().atf_decode_ex(q.data_ptr(), Kcache.data_ptr(), Vcache.data_ptr(), O.data_ptr(), B, Hq, Hkv, L, d, tab,
+                                   C.byref(o) if o is not None else None, _raw_stream(q)))
     if on_host:
         return (_to_pinned_host(O), _to_pinned_host(lse)) if return_lse else _to_pinned_host(O)
     return (O, lse) if return_lse else O
