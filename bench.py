@@ -428,7 +428,7 @@ def run_ours(args):
                      # DRAM bytes of one launch: ncu capture at N = 32768 (511 MB) scaled by N (traffic is the
                      # repacked Q/K, V and O once each, linear in N)
                      "traffic": 511.7e6 * wl.N / 32768 if wl.name == "llama-3.2-3b" else None,
-                     "kernel": "atf_prefill_pipe_kernel (+ schedule and 2 repack launches, <1% of the time)",
+                     "kernel": "atf_prefill_pipe_kernel (+ one pre-pass launch, <1% of the time)",
                      "peak_source": f"{pk['source']} sustained bf16 GEMM"},
         "roofline_decode": {"bound": "hbm", "achieved": dbytes / (dec_grp_us * 1e-6) / 1e9, "peak": pk["hbm_gbs"],
                             "unit": "GB/s", "frac": dbytes / (dec_grp_us * 1e-6) / 1e9 / pk["hbm_gbs"],
@@ -441,7 +441,7 @@ def run_ours(args):
         "e2e": {"value": executed / (e2e_ms * 1e-3) / 1e12, "unit": "TFLOP/s", "ms": e2e_ms,
                 "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                 "what": "atf_prefill on pinned host tensors = the C call atf_prefill_host: H2D of Q,K,V, kernels and D2H of O,LSE, overlapped chunk by chunk (16K rows) on three streams"},
-        "gpu_launches": 7 * args.steps,  # per step: 2 rope + schedule + 2 repack + prefill + decode
+        "gpu_launches": 5 * args.steps,  # per step: 2 rope + pre-pass + prefill + decode
         "clocks": clocks,
         "cpu_baseline": cpu,
     }

@@ -33,9 +33,9 @@
 // the rows over the whole 128 keys (the pair is live at the distance from the quarter's middle row
 // to the tile's middle column); the pairs a quarter does not keep are zeroed in its rows of the
 // CTA's copy of Q (pairs only die as the distance grows and the tiles are walked outwards from
-// the diagonal, so the zeroing is monotone).  A warp then finishes its 32 x 64 cells on the CUDA
-// cores: pairs in the MMA are taken back out of the cells beyond their window, pairs zeroed in Q
-// are added where live.  Coarse mode: depth = pairs live anywhere in the tile rounded up to 8,
+// the diagonal, so the zeroing is monotone).  A warp then finishes its 32 x 64 cells with small
+// products of its own (mma.sync): pairs in the MMA are taken back out of the cells beyond their window,
+// pairs zeroed in Q are added where live.  Coarse mode: depth = pairs live anywhere in the tile rounded up to 8,
 // everything on the diagonal tile, no per-cell work.
 //
 // Appended rows (App. C, "The interval itself"; Sec. 7.3): the tiles stay aligned at position 0 of the
@@ -534,7 +534,10 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
           //      One pair's masked term of 16 rows x 8 keys is ONE m16n8k16 product: the contraction runs over
           //      eight slots of two elements, slot j = key j; B holds the pair of key j in slot j only, A the
           //      pair of each row in the slots of the keys it takes.  S is brought in and put back in the
-          //      accumulator-fragment order. ----
+          //      accumulator-fragment order.  (Seven CUDA-core instructions a cell before: 24 heads x 8192 rows of 128
+          //      782 -> 698 us a layer step.  A step here still takes about twice a plain one: mma.sync waits beside
+          //      tcgen05, ~270 clocks an instruction when that pipe is full, K words wait for the S product's reads
+          //      of shared memory, and this code is seldom in the instruction cache.) ----
           const int p_lo = min(p_all, p_mid), p_hi = max(p_any, p_mid);
           if (p_lo < p_hi && zmax_w >= 0) {
             uint32_t q_next = 0u, ql_next = 0u;
