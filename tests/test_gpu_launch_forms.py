@@ -1,0 +1,54 @@
+"""Dispatch branches of the rotation (threads per row segment) and the prefill's overlapped launch, at their borders."""
+import numpy as np
+import pytest
+import torch
+
+import atf_inputs as gen
+from oracle import atf_oracle as orc
+
+pytestmark = pytest.mark.gpu
+
+
+# one, two, four and eight threads a segment (d = 128: from 18913, 9457, 4729 rows down), rows that do not fill a block,
+# fewer heads than threads
+@pytest.mark.parametrize("H,N,d", [(3, 18945, 128), (2, 18912, 128), (5, 9440, 128), (1, 4700, 128), (9, 33, 128), (3, 1, 64),
+                                   (3, 2501, 64), (1, 37889, 64)])
+def test_rope_threads_per_segment(H, N, d):
+    import paper_2608_02947_b200 as atf
+    X = gen.normal_bf16((1, H, N, d), 4242 + N)
+    _, theta = orc.window_table(5e5, d, 2.0, N)
+    ref = orc.rope_half_split(gen.to_f64(X), theta, pos0=77)  # rounded to bf16 once
+    out = gen.to_f64(atf.atf_rope(X.cuda(), theta, pos0=77))
+    # fp64 angles on both sides, one rounding: a tie may fall either way, one bf16 unit (2^-7 of the value at most)
+    assert np.all(np.abs(out - ref) <= 2.0 ** -7 * np.abs(ref) + 1e-30)
+    assert (out != ref).mean() < 1e-4
+    f = torch.randn((1, H, N, d), generator=torch.Generator().manual_seed(N))
+    ref = orc.rope_half_split(f.double().numpy(), theta, pos0=77, round_bf16=False)
+    out = atf.atf_rope_f32(f.cuda(), theta, pos0=77).double().cpu().numpy()
+    assert np.all(np.abs(out - ref) <= 2.0 ** -23 * np.abs(ref) + 1e-30)  # one rounding to fp32
+
+
+@pytest.mark.parametrize("split", [False, True])
+def test_prefill_back_to_back_and_captured(split):
+    """Calls that follow one another on one workspace, with new inputs each, give what each gives alone, also in a graph."""
+    import paper_2608_02947_b200 as atf
+    d, N, Nq = 128, 1000, 700
+    W, _ = atf.atf_window_table(5e5, d, 2.0, N)
+    gen_ = torch.Generator().manual_seed(5)
+    kind = torch.float32 if split else torch.bfloat16
+    cases = [[torch.randn((1, h, n, d), generator=gen_).to(t).cuda() for h, n, t in ((6, Nq, kind), (2, N, kind), (2, N, torch.bfloat16))]
+             for _ in range(3)]
+    call = atf.atf_prefill_split if split else atf.atf_prefill
+    alone = []
+    for q, k, v in cases:
+        alone.append([t.clone() for t in call(q, k, v, table=W)])
+        torch.cuda.synchronize()
+    together = [call(q, k, v, table=W) for q, k, v in cases]
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        captured = [call(q, k, v, table=W) for q, k, v in cases]
+    g.replay()
+    torch.cuda.synchronize()
+    for got in (together, captured):
+        for a, b in zip(alone, got):
+            assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
