@@ -584,28 +584,33 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
               // row g8 + 8 j takes the key of slot t4 (t4 + 4) of block cb inside the window iff 8 (cb - j) >= u (u - 4)
               const int u = zw_lo + g8 - t4 - 64 * h - wp;
               const uint32_t kp = krow + ((2 * p) >> 6) * BLK_BYTES + (((((2 * p) & 63) >> 3) ^ g8) << 4) + ((2 * p) & 7) * 2;
+              uint32_t kk[8], kl[SPLIT ? 8 : 1];
 #pragma unroll
-              for (int c2 = 0; c2 < 4; ++c2) {  // 16 keys at a time: distances [zw_lo - c0 - 15, zw_hi - c0]
-                const int c0 = 64 * h + 16 * c2;
-                if (subtract ? zw_hi - c0 > wp : (zw_lo - c0 - 15 <= wp && zw_hi >= c0)) {  // warp-uniform
+              for (int cb = 0; cb < 8; ++cb) {
+                asm volatile("ld.shared.b32 %0, [%1];" : "=r"(kk[cb]) : "r"(kp + cb * 1024));
+                if (SPLIT) asm volatile("ld.shared.b32 %0, [%1];" : "=r"(kl[cb]) : "r"(kp + SM::TILE + cb * 1024));
+              }
+              // Two halves of 32 keys, each taken whole if any cell of it changes (warp-uniform).  Branches cost more here
+              // than the products they save: 24 heads x 8192 rows of 128 take 650 us a layer step so, 667 with no branch,
+              // 680 with one for every 16 keys, 785 for 16 keys x 16 rows, 910 for 8 keys x 16 rows.
 #pragma unroll
-                  for (int cb = 2 * c2; cb < 2 * c2 + 2; ++cb) {
-                    uint32_t kk, kl = 0u;
-                    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(kk) : "r"(kp + cb * 1024));
-                    if (SPLIT) asm volatile("ld.shared.b32 %0, [%1];" : "=r"(kl) : "r"(kp + SM::TILE + cb * 1024));
+              for (int c4 = 0; c4 < 2; ++c4) {
+                const int zhi = zw_hi - 64 * h - 32 * c4;  // the half's distances: [zhi - 62, zhi]
+                if (subtract ? zhi <= wp : (zhi - 62 > wp || zhi < 0)) continue;
 #pragma unroll
-                    for (int hf = 0; hf < 2; ++hf) {
-                      const int i0 = 8 * (cb - 2 * hf), i1 = i0 - 8;  // rows g8 and g8 + 8 of the half
-                      const bool m0 = (i0 >= u) != subtract, m1 = (i1 >= u) != subtract;
-                      const bool m2 = (i0 + 4 >= u) != subtract, m3 = (i1 + 4 >= u) != subtract;
-                      const uint32_t a0 = m0 ? qr[2 * hf] : 0u, a1 = m1 ? qr[2 * hf + 1] : 0u;
-                      const uint32_t a2 = m2 ? qr[2 * hf] : 0u, a3 = m3 ? qr[2 * hf + 1] : 0u;
-                      mma_16816(f[hf] + 4 * cb, a0, a1, a2, a3, kk & slot0, kk & slot4);
-                      if (SPLIT) {  // the other two products of the split scores
-                        mma_16816(f[hf] + 4 * cb, a0, a1, a2, a3, kl & slot0, kl & slot4);
-                        mma_16816(f[hf] + 4 * cb, m0 ? qrl[2 * hf] : 0u, m1 ? qrl[2 * hf + 1] : 0u, m2 ? qrl[2 * hf] : 0u,
-                                  m3 ? qrl[2 * hf + 1] : 0u, kk & slot0, kk & slot4);
-                      }
+                for (int cb = 4 * c4; cb < 4 * c4 + 4; ++cb) {
+#pragma unroll
+                  for (int hf = 0; hf < 2; ++hf) {
+                    const int i0 = 8 * (cb - 2 * hf), i1 = i0 - 8;  // rows g8 and g8 + 8 of the half
+                    const bool m0 = (i0 >= u) != subtract, m1 = (i1 >= u) != subtract;
+                    const bool m2 = (i0 + 4 >= u) != subtract, m3 = (i1 + 4 >= u) != subtract;
+                    const uint32_t a0 = m0 ? qr[2 * hf] : 0u, a1 = m1 ? qr[2 * hf + 1] : 0u;
+                    const uint32_t a2 = m2 ? qr[2 * hf] : 0u, a3 = m3 ? qr[2 * hf + 1] : 0u;
+                    mma_16816(f[hf] + 4 * cb, a0, a1, a2, a3, kk[cb] & slot0, kk[cb] & slot4);
+                    if (SPLIT) {  // the other two products of the split scores
+                      mma_16816(f[hf] + 4 * cb, a0, a1, a2, a3, kl[cb] & slot0, kl[cb] & slot4);
+                      mma_16816(f[hf] + 4 * cb, m0 ? qrl[2 * hf] : 0u, m1 ? qrl[2 * hf + 1] : 0u, m2 ? qrl[2 * hf] : 0u,
+                                m3 ? qrl[2 * hf + 1] : 0u, kk[cb] & slot0, kk[cb] & slot4);
                     }
                   }
                 }
