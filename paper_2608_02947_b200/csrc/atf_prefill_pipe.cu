@@ -277,7 +277,7 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         auto load_k = [&](int t) {
           const int g = g0 + t, ks = g % KS;
           if (!wait_or_abort(bar(B_KEMPTY + ks), ((g / KS) & 1) ^ 1, abortp)) return false;
-          const int nkb = PipeWord(__ldg(P.sched + 8 * t)).nkb;
+          const int nkb = PipeWord(ld_sched(P.sched + 8 * t)).nkb;
           mbar_expect_tx(bar(B_KFULL + ks), SM::QN * nkb * BLK_BYTES);
           for (int kb = 0; kb < nkb; ++kb) {
             tma_load_3d(sK + ks * SM::KSTAGE + kb * BLK_BYTES, &tmK, bar(B_KFULL + ks), kb * 64, (it - t) * T, bhk);
@@ -318,7 +318,7 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         if (!iok) fail_site = 20;
         for (int t = 0; t < nt && iok; ++t) {
           const int g = g0 + t, sb = g & 1, ks = g % KS;
-          const int natoms = PipeWord(__ldg(P.sched + 8 * t)).natoms;
+          const int natoms = PipeWord(ld_sched(P.sched + 8 * t)).natoms;
           iok = wait_or_abort(bar(B_KFULL + ks), (g / KS) & 1, abortp);
           // both softmax groups hold S(g - 2) in registers: its buffer may be written again
           if (iok && g >= 2) iok = wait_or_abort(bar(B_SREAD + sb), ((g >> 1) - 1) & 1, abortp);
@@ -443,7 +443,7 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         }
       };
       const uint32_t* sched = P.sched + 2 * wq + h;
-      uint32_t e_cur = __ldg(sched);  // schedule word of the step at hand; the next one is fetched a step ahead
+      uint32_t e_cur = ld_sched(sched);  // schedule word of the step at hand; the next one is fetched a step ahead
       int p_mid = PipeWord(e_cur).p_mid;
       if constexpr (SPLIT) {
         if (MODE == ATF_MODE_EXACT) {
@@ -479,7 +479,7 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
           const int g = g0 + t, sb = g & 1, ks = g % KS;
           const PipeWord E(e_cur);
           if (!E.plain) break;
-          const uint32_t e_next = t + 1 < nt ? __ldg(sched + 8 * (t + 1)) : 0u;
+          const uint32_t e_next = t + 1 < nt ? ld_sched(sched + 8 * (t + 1)) : 0u;
           const int p_all = E.p_all, natoms = E.natoms;
           const int p_mid_next = PipeWord(e_next).p_mid;
           if (!wait_or_abort(bar(B_SFULL + sb), (g >> 1) & 1, abortp)) { ok = false; fail_site = 31; break; }
@@ -517,7 +517,7 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         const int zrow = dt * T + row;             // distance from this row to column 0 of the key tile
         const int zmax_w = dt * T + 32 * wq + 31 - 64 * h;  // over the warp's 32 x 64 cells
         const PipeWord E(e_cur);
-        const uint32_t e_next = t + 1 < nt ? __ldg(sched + 8 * (t + 1)) : 0u;
+        const uint32_t e_next = t + 1 < nt ? ld_sched(sched + 8 * (t + 1)) : 0u;
         const int p_all = E.p_all, p_any = E.p_any, natoms = E.natoms;
         const int p_mid_next = PipeWord(e_next).p_mid;
         const uint32_t tS = tmem_base + sb * T + 64 * h + lane_off;

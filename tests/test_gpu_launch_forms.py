@@ -52,3 +52,45 @@ def test_prefill_back_to_back_and_captured(split):
     for got in (together, captured):
         for a, b in zip(alone, got):
             assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
+
+
+@pytest.mark.parametrize("split", [False, True])
+def test_prefill_other_schedule_in_each_call(split):
+    """Calls on one workspace whose band schedules differ (table, mode, lengths), Q rotated in place right before each: the
+    words that the call before left, or a Q read too early, would show as other bits."""
+    import paper_2608_02947_b200 as atf
+    d = 128
+    rope = atf.atf_rope_f32 if split else atf.atf_rope
+    call = atf.atf_prefill_split if split else atf.atf_prefill
+    kind = torch.float32 if split else torch.bfloat16
+    gen_ = torch.Generator().manual_seed(6)
+    forms = [(1700, 1700, 2.0, atf.ATF_MODE_EXACT), (1000, 300, None, atf.ATF_MODE_EXACT), (1700, 900, 0.5, atf.ATF_MODE_COARSE),
+             (1700, 1700, 0.25, atf.ATF_MODE_EXACT), (129, 129, 2.0, atf.ATF_MODE_COARSE), (1700, 1700, None, atf.ATF_MODE_EXACT)]
+    cases = []
+    for N, Nq, k, mode in forms:
+        W, theta = atf.atf_window_table(5e5, d, k or 2.0, N)
+        q, key, v = [torch.randn((1, h, n, d), generator=gen_).to(t).cuda()
+                     for h, n, t in ((6, Nq, kind), (2, N, kind), (2, N, torch.bfloat16))]
+        cases.append((q, key, v, None if k is None else W, theta, N - Nq, mode))
+
+    def step(q, key, v, W, theta, pos0, mode):
+        q = q.clone()
+        return call(rope(q, theta, pos0=pos0), key, v, table=W, mode=mode)
+
+    alone = []
+    for c in cases:
+        alone.append([t.clone() for t in step(*c)])
+        torch.cuda.synchronize()
+    order = [0, 1, 2, 3, 4, 5, 3, 0, 4, 1, 5, 2]
+    for _ in range(3):
+        together = [(i, step(*cases[i])) for i in order]
+        torch.cuda.synchronize()
+        for i, got in together:
+            assert torch.equal(alone[i][0], got[0]) and torch.equal(alone[i][1], got[1])
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        captured = [(i, step(*cases[i])) for i in order]
+    g.replay()
+    torch.cuda.synchronize()
+    for i, got in captured:
+        assert torch.equal(alone[i][0], got[0]) and torch.equal(alone[i][1], got[1])
