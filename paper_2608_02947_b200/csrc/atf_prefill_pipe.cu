@@ -533,11 +533,14 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
           //      are zero in Q and live somewhere in the block: add their term inside the window.
           //      One pair's masked term of 16 rows x 8 keys is ONE m16n8k16 product: the contraction runs over
           //      eight slots of two elements, slot j = key j; B holds the pair of key j in slot j only, A the
-          //      pair of each row in the slots of the keys it takes.  S is brought in and put back in the
-          //      accumulator-fragment order.  (Seven CUDA-core instructions a cell before: 24 heads x 8192 rows of 128
-          //      782 -> 698 us a layer step.  A step here still takes about twice a plain one: mma.sync waits beside
-          //      tcgen05, ~270 clocks an instruction when that pipe is full, K words wait for the S product's reads
-          //      of shared memory, and this code is seldom in the instruction cache.) ----
+          //      pair of each row in the slots of the keys it takes.  The terms are summed from zero and added to S
+          //      once, rounded to nearest: mma.sync cuts a sum off, and onto S itself that cost up to a unit in the
+          //      last place of the score for every pair (LSE of the outlier inputs 5 % further from 64 bits).  S is
+          //      brought in 16 rows at a time for that (24 heads x 8192 rows of 128: 596 us, both halves at once 623,
+          //      before the pairs 659; summing onto S 586; seven CUDA-core instructions a cell, the first form, 704).
+          //      A step here still takes about twice a plain one: mma.sync waits beside tcgen05, ~270 clocks an
+          //      instruction when that pipe is full, K words wait for the S product's reads of shared memory, and this
+          //      code is seldom in the instruction cache. ----
           const int p_lo = min(p_all, p_mid), p_hi = max(p_any, p_mid);
           if (p_lo < p_hi && zmax_w >= 0) {
             uint32_t q_next = 0u, ql_next = 0u;
@@ -556,15 +559,8 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             fetch_q(p_lo);
             if (!wait_or_abort(bar(B_KFULL + ks), (g / KS) & 1, abortp)) { ok = false; fail_site = 32; break; }
             float f[2][32];  // rows 16 hf + {lane / 4, lane / 4 + 8}, keys 64h + 8 cb + 2 (lane % 4) + {0, 1}
-            if (s_valid) {
-              tc_ld_frag64(tS, f[0]);
-              tc_ld_frag64(tS + (16u << 16), f[1]);
-              tc_wait_ld();
-            } else {
 #pragma unroll
-              for (int e = 0; e < 32; ++e) f[0][e] = f[1][e] = 0.f;
-              s_valid = true;
-            }
+            for (int e = 0; e < 32; ++e) f[0][e] = f[1][e] = 0.f;
             const int g8 = lane >> 2, t4 = lane & 3;
             const uint32_t slot0 = g8 == t4 ? 0xFFFFFFFFu : 0u, slot4 = g8 == t4 + 4 ? 0xFFFFFFFFu : 0u;
             const int zw_lo = dt * T + wq * 32, zw_hi = zw_lo + 31;  // zrow over the warp's rows
@@ -591,8 +587,9 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 if (SPLIT) asm volatile("ld.shared.b32 %0, [%1];" : "=r"(kl[cb]) : "r"(kp + SM::TILE + cb * 1024));
               }
               // Two halves of 32 keys, each taken whole if any cell of it changes (warp-uniform).  Branches cost more here
-              // than the products they save: 24 heads x 8192 rows of 128 take 650 us a layer step so, 667 with no branch,
-              // 680 with one for every 16 keys, 785 for 16 keys x 16 rows, 910 for 8 keys x 16 rows.
+              // than the products they save (measured with S itself as the sum): 24 heads x 8192 rows of 128 took 650 us a
+              // layer step so, 667 with no branch, 680 with one for every 16 keys, 785 for 16 keys x 16 rows, 910 for
+              // 8 keys x 16 rows.
 #pragma unroll
               for (int c4 = 0; c4 < 2; ++c4) {
                 const int zhi = zw_hi - 64 * h - 32 * c4;  // the half's distances: [zhi - 62, zhi]
@@ -616,8 +613,22 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 }
               }
             }
-            tc_st_frag64(tS, f[0]);
-            tc_st_frag64(tS + (16u << 16), f[1]);
+#pragma unroll
+            for (int hf = 0; hf < 2; ++hf) {
+              if (s_valid) {
+                float sf[32];
+                tc_ld_frag64(tS + ((uint32_t)(16 * hf) << 16), sf);
+                tc_wait_ld();
+#pragma unroll
+                for (int e = 0; e < 32; e += 2) {
+                  const float2 v = __fadd2_rn(make_float2(f[hf][e], f[hf][e + 1]), make_float2(sf[e], sf[e + 1]));
+                  f[hf][e] = v.x;
+                  f[hf][e + 1] = v.y;
+                }
+              }
+              tc_st_frag64(tS + ((uint32_t)(16 * hf) << 16), f[hf]);
+            }
+            s_valid = true;
             tc_wait_st();
           }
         }
