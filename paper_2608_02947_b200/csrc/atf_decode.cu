@@ -93,8 +93,8 @@ __device__ __forceinline__ float ex2f(float x) {
 
 // The last block of a (batch, KV head) merges the partials of all splits by their log-sum-exp: one warp per head.  What
 // this costs is round trips to L2, so every load that can be in flight is: the (m, l) of up to 128 splits in one round
-// (lanes across the splits), then the outputs of MERGE_BATCH splits a round (lanes across the columns; past the last
-// split the loads repeat it with weight 0, because a remainder loop would pay a round trip for each split).
+// (lanes across the splits), then the outputs of MERGE_BATCH splits a round (lanes across the columns; loads past the last
+// split are left out one by one, because a remainder loop would pay a round trip for each split).
 constexpr int MERGE_BATCH = 16;
 template <int D, int NWARPS>
 __device__ __forceinline__ void merge_splits(const DecodeParams& P, int64_t grp, int64_t hq0, int warp, int lane) {
@@ -133,14 +133,15 @@ __device__ __forceinline__ void merge_splits(const DecodeParams& P, int64_t grp,
       float f[MERGE_BATCH], o[MERGE_BATCH][D / 32];
 #pragma unroll
       for (int i = 0; i < MERGE_BATCH; ++i) {
-        const float* src = base + min(s0 + i, ns - 1) * step;
-        f[i] = __ldcg(src);
+        const bool in = s0 + i < ns;
+        const float* src = base + (s0 + i) * step;
+        f[i] = in ? __ldcg(src) : -INFINITY;
 #pragma unroll
-        for (int c = 0; c < D / 32; ++c) o[i][c] = __ldcg(src + 2 + c * 32 + lane);
+        for (int c = 0; c < D / 32; ++c) o[i][c] = in ? __ldcg(src + 2 + c * 32 + lane) : 0.f;
       }
 #pragma unroll
       for (int i = 0; i < MERGE_BATCH; ++i) {
-        const float w = s0 + i < ns ? ex2f(f[i] - Ms) : 0.f;
+        const float w = ex2f(f[i] - Ms);
 #pragma unroll
         for (int c = 0; c < D / 32; ++c) acc[c] = fmaf(w, o[i][c], acc[c]);
       }

@@ -59,3 +59,21 @@ def test_scratch_for_one_split():
         assert lib.atf_decode_ex(*p, B, Hq, Hkv, L, d, tab, C.byref(opts), C.c_void_p(torch.cuda.current_stream().cuda_stream)) == code
     torch.cuda.synchronize()
     _check(O, None, ref)
+
+
+@pytest.mark.parametrize("L", [700, 1000, 2100])
+def test_infinite_value_stays_in_its_column(L):
+    """An infinite element of V makes its output column infinite and no other (11, 16 and more splits, in the last one too)."""
+    import paper_2608_02947_b200 as atf
+    q, K, V, W = _case(1, 6, 2, 128, L, 41)
+    q, K, V = q.cuda(), K.cuda(), V.cuda()
+    for cache in (K, atf.atf_kcache_pack(K)):
+        plain = atf.atf_decode(q, cache, V, table=W)
+        for key in (3, L // 2, L - 1):
+            v = V.clone()
+            v[0, 0, key, 5] = float("inf")
+            v[0, 0, key, 77] = -float("inf")
+            want = plain.clone()
+            want[0, :3, 5] = float("inf")
+            want[0, :3, 77] = -float("inf")
+            assert torch.equal(atf.atf_decode(q, cache, v, table=W), want), key
