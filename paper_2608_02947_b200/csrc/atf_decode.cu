@@ -949,29 +949,37 @@ atf_status launch_decode_tiles(const CUtensorMap& tmV, const DecodeParams& P, co
 atf_status atf_validate_table(const char* who, const int64_t* table, int d, int64_t N, AtfTable* out);
 
 // Splits of a (batch, KV head) over which a launch deals its `ntiles` tiles.  In units of one tile of a CTA that shares
-// its SM with another (about 1 us; alone on the SM it takes 3/4 of that), a launch costs
-//   the tiles a CTA walks, for each round of CTAs an SM runs (two at a time), + 14 for every round after the first
-//   (prologue, first loads, partials: 240 us in one round against 246 in two and 289 in four, eight sequences of 128K)
+// its SM with another (1 to 1.5 us; alone on the SM it takes 3/4 of that), a launch costs
+//   the tiles a CTA walks, for each round of CTAs an SM runs (two at a time), + 8 and 0.3 a tile, at most 14, for the
+//   second round and 4 for each further one (prologue, first loads, partials; later rounds run into one another)
 //   + the merge: a round trip to L2 for every MERGE_BATCH splits and every DEC_WARPS heads.
-// Measured, d = 128, 24/8 heads, the rule this replaced (at least 512 keys a split, fullest last wave) -> this one:
-// 512 keys 18.7 -> 8.2 us, 2048 keys 18.0 -> 10.2, 4096 keys 17.7 -> 12.6; two sequences of 32K 63 -> 50 us, eight
-// 151 -> 128 us.  Of equal costs the fewest splits are taken.
+// Over 1077 shapes (1 to 8000 groups, 300 to 150000 keys, both layouts) with every split count timed, the choice is 0.6 %
+// from the fastest one in the mean; the rule before it, which stopped at two rounds, 5 % (320 groups of 16384 keys, rows:
+// one split 671 us, nine 439), the one before that (at least 512 keys a split, fullest last wave) 16 %.
+// DEC_MAX_ROUNDS bounds search and scratch: past it more splits gained nothing at any shape.
+constexpr int DEC_SMS = 148, DEC_MAX_ROUNDS = 12;
+static int64_t decode_most_splits(int64_t groups, int64_t ntiles) {
+  return std::min<int64_t>(ntiles, std::max<int64_t>(1, DEC_MAX_ROUNDS * 2 * DEC_SMS / groups));
+}
 static int decode_splits(int64_t groups, int heads, int64_t ntiles) {
-  constexpr int SMS = 148;
-  const int64_t most = std::min<int64_t>(ntiles, std::max<int64_t>(1, 4 * SMS / groups));
+  const int64_t most = decode_most_splits(groups, ntiles);
   double best = 0.0;
-  int best_ns = 0;
-  for (int64_t ns = 1; ns <= most; ++ns) {
-    const int64_t per_sm = (groups * ns + SMS - 1) / SMS;
-    const double tiles = (double)((ntiles + ns - 1) / ns);
-    const double cost = tiles * ((double)(per_sm / 2) + 0.75 * (double)(per_sm & 1)) + 14.0 * (double)((per_sm - 1) / 2) +
+  int64_t best_ns = 0;
+  // Of the counts with equal tiles a split the fewest splits cost least: only those are looked at.
+  for (int64_t ns = 1; ns <= most;) {
+    const int64_t per_sm = (groups * ns + DEC_SMS - 1) / DEC_SMS, later = (per_sm - 1) / 2;
+    const int64_t tiles = (ntiles + ns - 1) / ns;
+    const double rounds = later ? std::min(14.0, 8.0 + 0.3 * (double)tiles) + 4.0 * (double)(later - 1) : 0.0;
+    const double cost = (double)tiles * ((double)(per_sm / 2) + 0.75 * (double)(per_sm & 1)) + rounds +
                         (double)((ns + MERGE_BATCH - 1) / MERGE_BATCH * ((heads + DEC_WARPS - 1) / DEC_WARPS));
     if (best_ns == 0 || cost < best) {
       best = cost;
-      best_ns = (int)ns;
+      best_ns = ns;
     }
+    if (tiles == 1) break;
+    ns = (ntiles + tiles - 2) / (tiles - 1);
   }
-  return best_ns;
+  return (int)best_ns;
 }
 
 // The least scratch a call is taken with (fewer splits than decode_splits asks for where it holds no more).
@@ -982,9 +990,10 @@ static size_t decode_ws_least(int B, int Hq, int Hkv, int64_t L, int d) {
   partials = (partials + 255) & ~(size_t)255;
   return ATF_WS_HEADER + partials;
 }
+// Room for any split count a call may take: it does not fall as L grows, so that one size serves a whole generation.
 size_t atf_decode_workspace_bytes(int B, int Hq, int Hkv, int64_t L, int d) {
   const int64_t kt = DEC_WARPS * (DEC_TILE_BYTES / (d * 2));
-  const size_t partials = (size_t)B * Hq * decode_splits((int64_t)B * Hkv, std::max(1, Hq / Hkv), (L + kt - 1) / kt) * (d + 2) * sizeof(float);
+  const size_t partials = (size_t)B * Hq * decode_most_splits((int64_t)B * Hkv, (L + kt - 1) / kt) * (d + 2) * sizeof(float);
   return std::max(decode_ws_least(B, Hq, Hkv, L, d), ATF_WS_HEADER + ((partials + 255) & ~(size_t)255));
 }
 

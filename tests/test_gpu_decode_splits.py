@@ -77,3 +77,27 @@ def test_infinite_value_stays_in_its_column(L):
             want[0, :3, 5] = float("inf")
             want[0, :3, 77] = -float("inf")
             assert torch.equal(atf.atf_decode(q, cache, v, table=W), want), key
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,d,L,least,most", [
+    (40, 24, 8, 128, 4096, 3, 8),    # 320 groups: one split each would leave 24 CTAs to walk 64 tiles on an idle GPU (181 us, 136 with 5)
+    (75, 28, 4, 128, 8192, 4, 12),   # 300 groups (330 us with one split, 233 with 7)
+    (51, 28, 4, 128, 65536, 3, 17),  # 204 groups, long contexts
+    (1, 24, 8, 128, 512, 8, 8)])
+def test_split_count(B, Hq, Hkv, d, L, least, most):
+    """Splits that a call takes: as many slots of its scratch are written, and its size does not fall as L grows."""
+    import paper_2608_02947_b200 as atf
+    size = [atf.atf_workspace_bytes(1, B, Hq, Hkv, n, d) for n in (1, L // 2, L, 2 * L, (2 ** 31 - 1) // d)]
+    assert size == sorted(size)
+    ws = torch.zeros(size[2], dtype=torch.uint8, device="cuda")
+    q = torch.randn((B, Hq, d), device="cuda").to(torch.bfloat16)
+    K = torch.randn((1, 1, L, d), device="cuda").to(torch.bfloat16).expand(B, Hkv, L, d).contiguous()
+    opts = atf.binding._Opts()
+    opts.workspace, opts.workspace_bytes = ws.data_ptr(), size[2]
+    O = torch.empty_like(q)
+    p = [C.c_void_p(t.data_ptr()) for t in (q, K, K, O)]
+    assert atf.lib().atf_decode_ex(*p, B, Hq, Hkv, L, d, None, C.byref(opts), C.c_void_p(torch.cuda.current_stream().cuda_stream)) == 0
+    part = ws[HEADER:].view(torch.float32)
+    written = int(part.nonzero().max()) + 1
+    splits = -(-written // (B * Hq * (d + 2)))
+    assert least <= splits <= most
