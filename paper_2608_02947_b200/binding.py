@@ -194,9 +194,15 @@ def _table_ptr(table, d):
 _ws = None
 
 
-@functools.lru_cache(maxsize=256)
 def atf_workspace_bytes(op, B, Hq, Hkv, N, d):
     return int(lib().atf_workspace_bytes(op, B, Hq, Hkv, N, d))
+
+
+@functools.lru_cache(maxsize=256)
+def _decode_scratch(B, Hq, Hkv, d):
+    """Workspace of a decode at any context length (the size does not fall as the length grows): the length of a generation
+    changes with every call, its scratch does not."""
+    return atf_workspace_bytes(ATF_OP_DECODE, B, Hq, Hkv, (2 ** 31 - 1) // max(d, 1), d)
 
 
 def ensure_workspace(nbytes, device):
@@ -473,7 +479,7 @@ def atf_decode(q, Kcache, Vcache, table=None, mode=ATF_MODE_EXACT, kept_terms=No
         O = torch.empty_like(q)
     lse = torch.empty((B, Hq), dtype=torch.float32, device=q.device) if return_lse else None
     dev = _one_device(q, Kcache, Vcache, O, kept_terms, rope_tables.buf if rope_tables is not None else None)
-    ensure_workspace(atf_workspace_bytes(ATF_OP_DECODE, B, Hq, Hkv, L, d), q.device)
+    ensure_workspace(_decode_scratch(B, Hq, Hkv, d), q.device)
     tab, _keep = _table_ptr(table, d)
     o = _opts(mode, kept_terms, lse, k_layout, kcache_groups=Kcache if k_layout == ATF_KLAYOUT_GROUPS else None)
     if rope_tables is not None:

@@ -88,13 +88,30 @@ __global__ void __launch_bounds__(ROPE_THREADS) atf_rope_kernel(T* __restrict__ 
     store8(row, olo);
     store8(row + H, ohi);
   };
-  const int64_t head = N * D;
-  T* row = X + ((int64_t)(threadIdx.x / SEGS) * N + n) * D + c * 8;
-  for (int bh = threadIdx.x / SEGS; bh < BH; bh += HL, row += HL * head) {
-    float lo[8], hi[8];
-    load8(row, lo);
-    load8(row + H, hi);
+  // this block's share of the heads: every (HL * gridDim.y)-th, the next one's row on its way while this one is rotated
+  const int64_t step = (int64_t)HL * gridDim.y;
+  int64_t bh = (int64_t)blockIdx.y * HL + threadIdx.x / SEGS;
+  if (bh >= BH) return;
+  T* row = X + (bh * N + n) * D + c * 8;
+  float lo[8], hi[8];
+  load8(row, lo);
+  load8(row + H, hi);
+  while (true) {
+    T* next = row + step * N * D;
+    bh += step;
+    float lo2[8], hi2[8];
+    if (bh < BH) {
+      load8(next, lo2);
+      load8(next + H, hi2);
+    }
     rotate(row, lo, hi);
+    if (bh >= BH) break;
+    row = next;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      lo[i] = lo2[i];
+      hi[i] = hi2[i];
+    }
   }
 }
 

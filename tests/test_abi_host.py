@@ -166,3 +166,12 @@ def test_rope_tables_validation_without_a_device(atf):
     assert b"needs" in lib.atf_last_error()
     th[7] = 0.0
     assert lib.atf_rope_tables(th, 128, 0, 1024, fake, 1 << 20, None) == 1            # theta must be positive
+
+
+def test_workspace_bytes_refuses_other_types_after_a_call():
+    """The size of a shape asked for once does not answer for an argument that the C call does not take."""
+    import paper_2608_02947_b200 as atf
+    for op in (0, 1, 2):
+        assert atf.atf_workspace_bytes(op, 1, 24, 8, 4096, 128) > 0
+        with pytest.raises(C.ArgumentError):
+            atf.atf_workspace_bytes(op, 1, 24, 8, 4096.0, 128)

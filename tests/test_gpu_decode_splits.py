@@ -101,3 +101,20 @@ def test_split_count(B, Hq, Hkv, d, L, least, most):
     written = int(part.nonzero().max()) + 1
     splits = -(-written // (B * Hq * (d + 2)))
     assert least <= splits <= most
+
+
+def test_one_scratch_for_a_generation():
+    """The binding's workspace does not change while a context grows token by token or by leaps."""
+    import paper_2608_02947_b200 as atf
+    torch.cuda.synchronize()
+    atf.binding._ws = None  # the next call binds a new one
+    B, Hq, Hkv, d = 1, 24, 8, 128
+    K = torch.randn((B, Hkv, 20000, d), device="cuda").to(torch.bfloat16)
+    q = torch.randn((B, Hq, d), device="cuda").to(torch.bfloat16)
+    seen = set()
+    for L in (60, 61, 65, 700, 5000, 20000, 300):
+        k = K[:, :, :L].contiguous()
+        atf.atf_decode(q, k, k)
+        seen.add((atf.binding._ws.data_ptr(), atf.binding._ws.numel()))
+    torch.cuda.synchronize()
+    assert len(seen) == 1
