@@ -1,6 +1,8 @@
 // atf_rope: half-split rotary embedding in place (Sec. 3.1).  Memory-bound elementwise pass;
 // the angle pos*theta_r, its sine/cosine and the rotation are evaluated in fp64 so that the
 // result is the correctly rounded bf16 of the exact rotation even at positions ~2^20.
+#include <algorithm>
+
 #include "atf_common.cuh"
 
 struct RopeTheta {
@@ -43,8 +45,10 @@ __device__ __forceinline__ void store8(float* p, const double (&v)[8]) {
 // 128: 276 us, 5.8 TB/s).  For short ones HL fills the GPU; spreading the heads over blocks instead, each with the
 // angles evaluated again, made the fp64 pipe the bound: 24 heads x 8192 x 128 23.2 -> 18.0 us, 8 heads 15.3 -> 8.5 us,
 // 24 heads x 2048 12.8 -> 7.1 us.
+// SPREAD: the heads are dealt over gridDim.y blocks as well, for rows too few to fill the GPU.
+// PRE: the next head's segment is loaded before this one is stored, for fp32 data that L2 does not hold.
 constexpr int ROPE_THREADS = 256;
-template <int D, int HL, typename T>
+template <int D, int HL, typename T, bool SPREAD = false, bool PRE = false>
 __global__ void __launch_bounds__(ROPE_THREADS) atf_rope_kernel(T* __restrict__ X, int BH, int64_t N, int64_t pos0,
                                                                 const __grid_constant__ RopeTheta theta) {
   constexpr int H = D / 2;
@@ -88,45 +92,71 @@ __global__ void __launch_bounds__(ROPE_THREADS) atf_rope_kernel(T* __restrict__ 
     store8(row, olo);
     store8(row + H, ohi);
   };
-  // this block's share of the heads: every (HL * gridDim.y)-th, the next one's row on its way while this one is rotated
-  const int64_t step = (int64_t)HL * gridDim.y;
-  int64_t bh = (int64_t)blockIdx.y * HL + threadIdx.x / SEGS;
-  if (bh >= BH) return;
-  T* row = X + (bh * N + n) * D + c * 8;
+  const int64_t head = N * D;
+  const int lane = threadIdx.x / SEGS;
+  const int first = SPREAD ? (int)blockIdx.y * HL + lane : lane, step = SPREAD ? HL * (int)gridDim.y : HL;
+  T* row = X + ((int64_t)first * N + n) * D + c * 8;
   float lo[8], hi[8];
-  load8(row, lo);
-  load8(row + H, hi);
-  while (true) {
-    T* next = row + step * N * D;
-    bh += step;
-    float lo2[8], hi2[8];
-    if (bh < BH) {
-      load8(next, lo2);
-      load8(next + H, hi2);
-    }
-    rotate(row, lo, hi);
-    if (bh >= BH) break;
-    row = next;
+  if constexpr (PRE) {
+    if (first >= BH) return;
+    load8(row, lo);
+    load8(row + H, hi);
+  }
+  for (int bh = first; bh < BH; bh += step, row += step * head) {
+    if constexpr (PRE) {
+      float lo2[8], hi2[8];
+      if (bh + step < BH) {
+        load8(row + step * head, lo2);
+        load8(row + step * head + H, hi2);
+      }
+      rotate(row, lo, hi);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      lo[i] = lo2[i];
-      hi[i] = hi2[i];
+      for (int i = 0; i < 8; ++i) {
+        lo[i] = lo2[i];
+        hi[i] = hi2[i];
+      }
+    } else {
+      load8(row, lo);
+      load8(row + H, hi);
+      rotate(row, lo, hi);
     }
   }
 }
 
 // Threads per row segment: one as long as that gives four blocks (fp32: eight, its rows are twice as long) for each SM, more
-// for shorter rows.
+// for shorter rows; more threads than heads (they share the angles' evaluation only) below two blocks.  Eight threads walk
+// at least every eighth head, one round trip to memory each; rows that do not give three blocks for each SM then have
+// their heads dealt over blocks too, each with the angles evaluated again (d = 128, bf16, us, without -> with: 192 heads x 1 row, the queries of a decode step, 13.2 -> 2.4; 1536 x 1 91 -> 2.9; 2048 x 33
+// 127 -> 9.3; 192 x 128 14.5 -> 4.4; 192 x 512 14.7 -> 10.5; 24 x 128 3.6 -> 2.6).
+// fp32 moves twice the bytes an angle and is bound by the loads in flight: the heads are dealt over twelve blocks for each SM
+// (192 heads x 512 20.6 -> 18, 100 x 1500 29 -> 26).  Past the 126 MB of L2 a thread waits for DRAM between its heads unless
+// the next one is on its way (192 heads x 2048 96 -> 69 us, 24 x 32768 200 -> 132, 24 x 131072 603 -> 504); smaller
+// data is slower so (24 x 8192 31.6 -> 33.0), and so is bf16 (24 x 131072 272 -> 306).
 template <int D, typename T>
 static void launch_rope(T* X, int BH, int64_t N, int64_t pos0, const RopeTheta& th, cudaStream_t s) {
-  int hl = 1;
+  constexpr bool F32 = sizeof(T) == 4;
   const auto blocks = [&](int lanes) { return (N + ROPE_THREADS / lanes / (D / 16) - 1) / (ROPE_THREADS / lanes / (D / 16)); };
-  while (hl < 8 && blocks(hl) < 2 * (int)sizeof(T) * 148) hl *= 2;
-  const unsigned g = (unsigned)blocks(hl);
-  if (hl == 1) atf_rope_kernel<D, 1, T><<<g, ROPE_THREADS, 0, s>>>(X, BH, N, pos0, th);
-  else if (hl == 2) atf_rope_kernel<D, 2, T><<<g, ROPE_THREADS, 0, s>>>(X, BH, N, pos0, th);
-  else if (hl == 4) atf_rope_kernel<D, 4, T><<<g, ROPE_THREADS, 0, s>>>(X, BH, N, pos0, th);
-  else atf_rope_kernel<D, 8, T><<<g, ROPE_THREADS, 0, s>>>(X, BH, N, pos0, th);
+  int hl = 1;
+  while (hl < 8 && blocks(hl) < (2 * hl > BH ? 2 : 2 * (int)sizeof(T)) * 148) hl *= 2;
+  const bool pre = F32 && (double)BH * (double)N * D * sizeof(T) > 126e6 && blocks(hl) >= 3 * 148;
+  if (F32 && !pre)
+    while (hl < 8 && 2 * hl <= BH) hl *= 2;
+  const unsigned g = (unsigned)blocks(hl), want = (F32 ? 12 : 3) * 148;
+  if (!pre && hl == 8 && BH > 8 && g < want) {
+    const unsigned gy = std::min(((unsigned)BH + 7) / 8, (want + g - 1) / g);
+    atf_rope_kernel<D, 8, T, true><<<dim3(g, gy), ROPE_THREADS, 0, s>>>(X, BH, N, pos0, th);
+    return;
+  }
+#define ATF_ROPE_LAUNCH(HL_)                                                                        \
+  do {                                                                                              \
+    if (pre) atf_rope_kernel<D, HL_, T, false, F32><<<g, ROPE_THREADS, 0, s>>>(X, BH, N, pos0, th);  \
+    else atf_rope_kernel<D, HL_, T><<<g, ROPE_THREADS, 0, s>>>(X, BH, N, pos0, th);                 \
+  } while (0)
+  if (hl == 1) ATF_ROPE_LAUNCH(1);
+  else if (hl == 2) ATF_ROPE_LAUNCH(2);
+  else if (hl == 4) ATF_ROPE_LAUNCH(4);
+  else ATF_ROPE_LAUNCH(8);
+#undef ATF_ROPE_LAUNCH
 }
 
 template <typename T>

@@ -94,3 +94,29 @@ def test_prefill_other_schedule_in_each_call(split):
     torch.cuda.synchronize()
     for i, got in captured:
         assert torch.equal(alone[i][0], got[0]) and torch.equal(alone[i][1], got[1])
+
+
+# heads dealt over blocks (few rows; a last block with fewer heads than threads; fp32 up to twelve blocks an SM), a last row
+# that does not fill a block, fp32 with the next head on its way (more than 126 MB; heads that do not divide by the threads)
+@pytest.mark.parametrize("B,H,N,d,f32", [(8, 24, 1, 128, False), (64, 28, 1, 64, False), (3, 67, 5, 128, False), (2, 9, 440, 64, False),
+                                         (8, 24, 1, 128, True), (3, 67, 5, 64, True), (5, 11, 700, 128, True), (1, 6, 9001, 64, True),
+                                         (2, 53, 2401, 128, True), (1, 3, 90001, 128, True)])
+def test_rope_heads_over_blocks(B, H, N, d, f32):
+    import paper_2608_02947_b200 as atf
+    _, theta = orc.window_table(5e5, d, 2.0, N)
+    X = torch.randn((B, H, N, d), generator=torch.Generator().manual_seed(N))
+    if not f32:
+        X = X.to(torch.bfloat16)
+    out = (atf.atf_rope_f32 if f32 else atf.atf_rope)(X.cuda(), theta, pos0=1234)
+    # a head at a time, as the oracle rotates it: fp64, one rounding (a tie may fall either way)
+    for b, h in {(0, 0), (0, H - 1), (B - 1, 0), (B - 1, H - 1), (B // 2, H // 2), (B - 1, min(8, H - 1))}:
+        ref = orc.rope_half_split(X[b, h].double().numpy(), theta, pos0=1234, round_bf16=not f32)
+        got = out[b, h].double().cpu().numpy()
+        assert np.all(np.abs(got - ref) <= 2.0 ** (-23 if f32 else -7) * np.abs(ref) + 1e-30)
+    # every head is rotated, and once: the length of a pair does not change
+    n = d // 2
+    was, now = X.cuda().double(), out.double()
+    was, now = was[..., :n] ** 2 + was[..., n:] ** 2, now[..., :n] ** 2 + now[..., n:] ** 2
+    assert torch.all((was - now).abs() <= 2.0 ** (-21 if f32 else -6) * was + 1e-30)
+    if N > 1:
+        assert not torch.equal(out[..., 1, :], X.cuda()[..., 1, :])
