@@ -403,15 +403,16 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       return r;
     };
     // This group's half of the pairs of the row, p = h H/2 + i: dims H-1-p and D-1-p, which are QW consecutive elements of
-    // each half row in falling order.  Rows that do not exist (before n0, from N on) are zero.
+    // each half row in falling order.  Rows that do not exist (before n0, from N on) are zero.  Ordinary loads: a caller may
+    // have O written over Q (the rows a CTA writes are those it alone has read).
     constexpr int QW = H / 2;
     auto load_q = [&](uint32_t (&w)[QW]) {
       const __nv_bfloat16* q = P.Q + qrow * D + (H - QW - h * QW);
       uint32_t x[QW / 2], y[QW / 2];
 #pragma unroll
       for (int i = 0; i < QW / 2; i += 4) {
-        *reinterpret_cast<uint4*>(x + i) = row_ok ? __ldg(reinterpret_cast<const uint4*>(q + 2 * i)) : make_uint4(0u, 0u, 0u, 0u);
-        *reinterpret_cast<uint4*>(y + i) = row_ok ? __ldg(reinterpret_cast<const uint4*>(q + H + 2 * i)) : make_uint4(0u, 0u, 0u, 0u);
+        *reinterpret_cast<uint4*>(x + i) = row_ok ? *reinterpret_cast<const uint4*>(q + 2 * i) : make_uint4(0u, 0u, 0u, 0u);
+        *reinterpret_cast<uint4*>(y + i) = row_ok ? *reinterpret_cast<const uint4*>(q + H + 2 * i) : make_uint4(0u, 0u, 0u, 0u);
       }
 #pragma unroll
       for (int i = 0; i < QW; ++i) w[i] = __byte_perm(x[(QW - 1 - i) >> 1], y[(QW - 1 - i) >> 1], (i & 1) ? 0x5410 : 0x7632);

@@ -120,3 +120,22 @@ def test_rope_heads_over_blocks(B, H, N, d, f32):
     assert torch.all((was - now).abs() <= 2.0 ** (-21 if f32 else -6) * was + 1e-30)
     if N > 1:
         assert not torch.equal(out[..., 1, :], X.cuda()[..., 1, :])
+
+
+@pytest.mark.parametrize("d,mode,outlier", [(128, 0, False), (128, 1, False), (64, 0, True), (128, 0, True)])
+def test_prefill_output_over_its_queries(d, mode, outlier):
+    """O written over Q, also where tiles are run twice (outlier logits read Q again)."""
+    import paper_2608_02947_b200 as atf
+    N, Nq = 1500, 1100
+    g = torch.Generator().manual_seed(d + mode)
+    Q, K, V = [torch.randn((2, h, n, d), generator=g) for h, n in ((6, Nq), (2, N), (2, N))]
+    W, theta = atf.atf_window_table(5e5, d, 2.0, N)
+    if outlier:
+        for t in (Q, K):
+            t[..., d // 2 - 4:d // 2] *= 8
+            t[..., d - 4:] *= 8
+    Q, K, V = (t.to(torch.bfloat16).cuda() for t in (Q, K, V))
+    O, lse = atf.atf_prefill(Q, K, V, table=W, mode=mode)
+    got, lse2 = atf.atf_prefill(Q, K, V, table=W, mode=mode, O=Q)
+    assert got.data_ptr() == Q.data_ptr()
+    assert torch.equal(got, O) and torch.equal(lse2, lse)
