@@ -35,7 +35,7 @@ HostPlan make_plan(int B, int Hq, int Hkv, int64_t N, int d, int64_t chunk_rows)
   // takes (see atf_prefill_chunk) and with it the last bit of a result
   const int64_t want = chunk_rows > 0 ? (chunk_rows + 127) / 128 * 128 : DEFAULT_CHUNK;
   p.chunk = std::min<int64_t>(want, N);
-  // workspace of one chunk call: header + repacked Q chunk + repacked K of up to N rows
+  // workspace of one chunk call (K reordered for up to N rows; the size counts Q as well, see atf_prefill_workspace_bytes)
   p.ws = align256(atf_prefill_workspace_bytes(B, Hq, Hkv, N, d));
   p.kv = align256((size_t)B * Hkv * N * d * 2);
   p.qbuf = align256((size_t)B * Hq * p.chunk * d * 2);

@@ -4,7 +4,7 @@
 // With a single query tile the 512 tensor-memory columns hold two S buffers, two P buffers and O, so
 // the chain "softmax -> O += P V -> next S -> softmax" is cut: S(t + 1) = Q K(t + 1)^T is computed
 // while the softmax groups work on S(t), and O += P(t) V runs whenever P(t) is stored.  Warp roles:
-//   warp 0      TMA producer: K (live 64-column blocks) and V tiles into three-stage rings of
+//   warp 0      TMA producer: K (live 64-column blocks) and V tiles into rings (stages: PipeSmem) of
 //               128-byte-swizzled shared memory;
 //   warp 1      issuer of S(t) = Q K(t)^T over the live depth (one thread, tcgen05.mma SS form);
 //   warp 2      issuer of O += P(t) V(t), half a tile at a time (one thread, TS form: P is read from
@@ -15,8 +15,9 @@
 // store them to shared memory in the column order of atf_prefill.cu.  A row of Q is read by one CTA only, so a pre-pass
 // that reorders it would move it twice more (8192 rows of 24 heads: 22 us of 700).  The split-precision mode keeps such
 // a pre-pass and loads Q by TMA: splitting fp32 rows here took longer (10001 rows: 1.21 against 1.19 ms).  Exact mode
-// holds a second, whole copy for the per-cell finish, where a pair fetched from global memory cost an L2 round trip
-// (8192 rows: 733 us against 685); at d = 128 that leaves two K stages, which long rows feel (131072 rows: + 1 %).
+// holds a second, whole copy for the per-cell finish, where a pair fetched from global memory costs an L2 round trip; at
+// d = 128 that leaves two K stages instead of three, which pays at every length (24 heads of 8192 rows 596 us against 636,
+// of 131072 rows 83.9 ms against 85.8).  Full attention, which finishes nothing, runs the coarse form (atf_prefill.cu).
 // The launch overlaps the end of the pre-pass (programmatic dependent launch): everything up to Q needs nothing of it.
 // The two threads of a row never meet in the common step: exponentials are taken against the
 // row's reference maximum from the diagonal tile (any reference gives the same softmax as long

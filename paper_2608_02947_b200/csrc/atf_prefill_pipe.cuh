@@ -1,5 +1,5 @@
 // Launch interface of the one-tile-per-CTA prefill pipeline (atf_prefill_pipe.cu); the host code of
-// atf_prefill.cu (validation, repacking, tensor maps) serves both pipelines.
+// atf_prefill.cu and atf_prefill_split.cu (validation, pre-pass, tensor maps) calls it.
 #pragma once
 
 #include "atf_common.cuh"
