@@ -215,6 +215,15 @@ def ensure_workspace(nbytes, device):
     return _ws
 
 
+def _ensure_decode_workspace(B, Hq, Hkv, L, d, device):
+    """A bound workspace with room for this call stays (a caller may have sized it and captured it in a graph); a new one has
+    room for every length to come."""
+    most = _decode_scratch(B, Hq, Hkv, d)
+    if _ws is None or _ws.device != device or (_ws.numel() < most and
+                                               _ws.numel() < atf_workspace_bytes(ATF_OP_DECODE, B, Hq, Hkv, L, d)):
+        ensure_workspace(most, device)
+
+
 def atf_rope(X, theta, pos0=0):
     """In-place half-split RoPE of X [B,H,N,d] (CUDA bf16) at positions pos0..pos0+N-1."""
     _dev_bf16(X, "X")
@@ -479,7 +488,7 @@ def atf_decode(q, Kcache, Vcache, table=None, mode=ATF_MODE_EXACT, kept_terms=No
         O = torch.empty_like(q)
     lse = torch.empty((B, Hq), dtype=torch.float32, device=q.device) if return_lse else None
     dev = _one_device(q, Kcache, Vcache, O, kept_terms, rope_tables.buf if rope_tables is not None else None)
-    ensure_workspace(_decode_scratch(B, Hq, Hkv, d), q.device)
+    _ensure_decode_workspace(B, Hq, Hkv, L, d, q.device)
     tab, _keep = _table_ptr(table, d)
     o = _opts(mode, kept_terms, lse, k_layout, kcache_groups=Kcache if k_layout == ATF_KLAYOUT_GROUPS else None)
     if rope_tables is not None:

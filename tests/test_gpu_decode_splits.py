@@ -118,3 +118,21 @@ def test_one_scratch_for_a_generation():
         seen.add((atf.binding._ws.data_ptr(), atf.binding._ws.numel()))
     torch.cuda.synchronize()
     assert len(seen) == 1
+
+
+def test_workspace_sized_by_the_caller_stays():
+    """A workspace of the size asked for one length is kept for calls of that length (and replaced for a longer one)."""
+    import paper_2608_02947_b200 as atf
+    B, Hq, Hkv, d, L = 1, 14, 2, 64, 1000
+    torch.cuda.synchronize()
+    atf.binding._ws = None
+    ws = atf.ensure_workspace(atf.atf_workspace_bytes(1, B, Hq, Hkv, L, d), "cuda:0")
+    K = torch.randn((B, Hkv, 8 * L, d), device="cuda").to(torch.bfloat16)
+    q = torch.randn((B, Hq, d), device="cuda").to(torch.bfloat16)
+    for n in (L, L - 1, 1):
+        k = K[:, :, :n].contiguous()
+        atf.atf_decode(q, k, k)
+        assert atf.binding._ws is ws
+    atf.atf_decode(q, K, K)
+    assert atf.binding._ws.numel() > ws.numel()
+    torch.cuda.synchronize()
