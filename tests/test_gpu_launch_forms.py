@@ -139,3 +139,30 @@ def test_prefill_output_over_its_queries(d, mode, outlier):
     got, lse2 = atf.atf_prefill(Q, K, V, table=W, mode=mode, O=Q)
     assert got.data_ptr() == Q.data_ptr()
     assert torch.equal(got, O) and torch.equal(lse2, lse)
+
+
+@pytest.mark.parametrize("N", [300, 14817])
+def test_prefill_and_decode_in_turn_on_one_workspace(N):
+    """The decode's partials lie where the next prefill's schedule is written: 300 layer steps give what the first one gave."""
+    import paper_2608_02947_b200 as atf
+    Hq, Hkv, d = 14, 2, 64
+    W, theta = atf.atf_window_table(1e6, d, 2.0, N)
+    table = atf.WindowTable(W)
+    g = torch.Generator(device="cuda").manual_seed(N)
+    Q, K, V = [torch.randn((1, h, N, d), generator=g, device="cuda").to(torch.bfloat16) for h in (Hq, Hkv, Hkv)]
+    cache = atf.new_kcache_groups(1, Hkv, N, d, "cuda")
+    atf.atf_rope(Q, theta)
+    atf.atf_rope(K, theta)
+    q = Q[:, :, -1].contiguous()
+
+    def step():
+        O, lse = atf.atf_prefill(Q, K, V, table=table, kcache_groups=cache)
+        return O, lse, atf.atf_decode(q, cache, V, table=table)
+
+    first = step()
+    other = torch.zeros((), dtype=torch.bool, device="cuda")
+    for _ in range(300):
+        for a, b in zip(first, step()):
+            other |= (a != b).any()
+    assert not other.item()
+    atf.binding.check_status()
