@@ -85,6 +85,19 @@ __device__ __forceinline__ void mma_bf16_16816(float (&c)[4], uint32_t a0, uint3
                : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
                : "r"(a0), "r"(0u), "r"(a2), "r"(0u), "r"(b0), "r"(b1));
 }
+// D (16x8, fp32) += A (16x16, bf16) * B (16x8, bf16)
+__device__ __forceinline__ void mma_bf16_full(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                              uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+// An 8x8 matrix of 16-bit elements spread over the warp (row lane / 4, columns 2 (lane % 4) + {0, 1}), transposed.
+__device__ __forceinline__ uint32_t movmatrix_trans(uint32_t v) {
+  uint32_t r;
+  asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(r) : "r"(v));
+  return r;
+}
 __device__ __forceinline__ float ex2f(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -499,7 +512,7 @@ atf_decode_kernel(const __grid_constant__ DecodeParams P, const __grid_constant_
 // halves of a key's group entry are stored swapped for keys with bit 2 set, which makes the
 // ldmatrix reads of the copied image free of bank conflicts without padding.  The V tile (rows of
 // the ordinary cache) comes by TMA with the 128-byte swizzle for the same reason.
-// Block = 4 consumer warps (a quarter of the tile each, the arithmetic of the row-layout kernel)
+// Block = 4 consumer warps (a quarter of the tile each, the row-layout kernel's steps with its products transposed)
 // + 1 producer warp (one thread issues the copies of the next tiles into a 3-stage ring; full and
 // empty mbarriers per stage, every wait bounded).
 // ------------------------------------------------------------------------------------------
@@ -510,9 +523,6 @@ constexpr int TL_STAGES = ATF_TL_STAGES;
 constexpr int TL_THREADS = (DEC_WARPS + 1) * 32;
 constexpr int TL_TILE_BYTES = 16384;
 constexpr int TL_STAGE_BYTES = 2 * TL_TILE_BYTES;
-#ifndef ATF_ROT_BATCH
-#define ATF_ROT_BATCH 2
-#endif
 constexpr int TL_ROT_BYTES = 1024;  // room for one row of the tile-level rotation table (keeps the stages 1 KiB aligned)
 constexpr int TL_SMEM = TL_STAGES * TL_STAGE_BYTES + 1024 /* alignment slack */ + 64 /* barriers */;
 __device__ __forceinline__ float2 lds_f2(uint32_t addr) {
@@ -521,12 +531,17 @@ __device__ __forceinline__ float2 lds_f2(uint32_t addr) {
   return v;
 }
 
-// One (dim r, dim r + h) pair of an unrotated key, turned by the angle a + b given as (cos, sin) of a and of b
-// (App. B: the rotation applied when the cache is read).  fp32, one rounding to bf16.
-__device__ __forceinline__ uint32_t rotate_pair(uint32_t v, float2 a, float2 b) {
-  const float c = fmaf(a.x, b.x, -a.y * b.y), s = fmaf(a.y, b.x, a.x * b.y);
-  const float x = __uint_as_float(v << 16), y = __uint_as_float(v & 0xffff0000u);
-  return pack_bf16x2(fmaf(x, c, -y * s), fmaf(y, c, x * s));
+// The (dim r, dim r + h) pair of two unrotated keys, turned by the angles a + b given as (cos, sin) of a, of the tile, and of
+// b, of each key in its tile (App. B: the rotation applied when the cache is read).  fp32, one rounding to bf16.
+__device__ __forceinline__ void rotate_pairs(uint32_t& v0, uint32_t& v1, float2 a, float2 bc, float2 bs) {
+  const float2 ax = make_float2(a.x, a.x), ay = make_float2(a.y, a.y), nay = make_float2(-a.y, -a.y);
+  const float2 c = __ffma2_rn(ax, bc, __fmul2_rn(nay, bs)), s = __ffma2_rn(ay, bc, __fmul2_rn(ax, bs));
+  const float2 ns = __fmul2_rn(s, make_float2(-1.f, -1.f));
+  const float2 x = make_float2(__uint_as_float(v0 << 16), __uint_as_float(v1 << 16));
+  const float2 y = make_float2(__uint_as_float(v0 & 0xffff0000u), __uint_as_float(v1 & 0xffff0000u));
+  const float2 xr = __ffma2_rn(x, c, __fmul2_rn(y, ns)), yr = __ffma2_rn(y, c, __fmul2_rn(x, s));
+  v0 = pack_bf16x2(xr.x, yr.x);
+  v1 = pack_bf16x2(xr.y, yr.y);
 }
 
 template <int D, int MODE, bool COUNT, bool ROT>
@@ -596,12 +611,14 @@ atf_decode_tiles_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_co
     }
   };
 
-  float oacc[NNT][4];
+  // Both products are taken transposed, so that the keys or the dims fill the 16 rows of an mma and the (up to 8) heads are
+  // its 8 columns: half the products and half the accumulators of the form with the heads as rows.
+  float oacc[NNT / 2][4];  // dims 16 np + g + {0, 0, 8, 8}, heads 2 t4 + {0, 1, 0, 1}
 #pragma unroll
-  for (int nt = 0; nt < NNT; ++nt)
+  for (int np = 0; np < NNT / 2; ++np)
 #pragma unroll
-    for (int e = 0; e < 4; ++e) oacc[nt][e] = 0.f;
-  float m_used = -INFINITY, l_part = 0.f;
+    for (int e = 0; e < 4; ++e) oacc[np][e] = 0.f;
+  float m_used[2] = {-INFINITY, -INFINITY}, l_part[2] = {0.f, 0.f};  // of heads 2 t4 and 2 t4 + 1
   unsigned long long cnt = 0;
 
   if (warp == DEC_WARPS) {
@@ -631,7 +648,7 @@ atf_decode_tiles_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_co
     }
   } else {
     // =============================== consumers ===============================
-    // A fragments of q: K step j contracts the 8 pairs of group j, each pair as (dim r, dim r + h)
+    // B fragments of q: K step j contracts the 8 pairs of group j, each pair as (dim r, dim r + h)
     uint32_t qa[NKS][2];
 #pragma unroll
     for (int j = 0; j < NKS; ++j) {
@@ -643,6 +660,23 @@ atf_decode_tiles_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_co
         qa[j][0] = (uint32_t)q16[ra] | ((uint32_t)q16[ra + H] << 16);
         qa[j][1] = (uint32_t)q16[rb] | ((uint32_t)q16[rb + H] << 16);
       }
+    }
+    // Rotate-at-read: (cos, sin) of the key-level angles of this lane's pairs and keys.  They are the same in every tile and
+    // stay in registers, which the transposed products leave room for; read through L1 for every tile and rotated by scalar
+    // arithmetic, 24 heads x 131072 keys took 86 us, now 74 (eight sequences of 32768: 201, now 154).
+    float2 kc[ROT ? NKS : 1][2][ROT ? NKG / 2 : 1], ksi[ROT ? NKS : 1][2][ROT ? NKG / 2 : 1];
+    if (ROT) {
+#pragma unroll
+      for (int j = 0; j < NKS; ++j)
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+#pragma unroll
+          for (int kp = 0; kp < NKG / 2; ++kp) {
+            const float2* src = P.rot_key + (8 * j + 4 * c + t4) * KT + warp * KB + 16 * kp + g;
+            const float2 k0 = __ldg(src), k1 = __ldg(src + 8);
+            kc[j][c][kp] = make_float2(k0.x, k1.x);
+            ksi[j][c][kp] = make_float2(k0.y, k1.y);
+          }
     }
     const int lm_i = lane >> 3, lm_r = lane & 7;
     // K: matrices (keys 0-7 first half), (keys 0-7 second half), (keys 8-15 first half), (keys 8-15 second half)
@@ -684,33 +718,27 @@ atf_decode_tiles_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_co
           r_lane[kg] = MODE == ATF_MODE_COARSE ? (r >= H ? H : (r & ~7)) : r;
         }
       }
-      float sc[NKG][4];
+      float sc[NKG / 2][4];  // keys 16 kp + g + {0, 0, 8, 8}, heads 2 t4 + {0, 1, 0, 1}
 #pragma unroll
-      for (int kg = 0; kg < NKG; ++kg)
+      for (int kp = 0; kp < NKG / 2; ++kp)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) sc[kg][e] = 0.f;
+        for (int e = 0; e < 4; ++e) sc[kp][e] = 0.f;
 
       // ---- S = q K^T: K step j = the 8 pairs of group j; a key with first live pair r keeps its first H - r pairs ----
       const int ngl = (H - rq_near + 7) >> 3;
-      // Rotate-at-read works on JB groups per branch, so that the table reads and the rotations of several
-      // groups overlap; a group beyond the fetched prefix holds stale bytes, which the masks below zero.
-      constexpr int JB = ROT ? ATF_ROT_BATCH : 1;
+      // Rotate-at-read works on JB groups per branch, so that the rotations of several groups overlap; a group beyond the
+      // fetched prefix holds stale bytes, which the masks below zero (131072 keys of 128 columns: one group 78 us, two 74,
+      // four 76; 50000 keys of 64: 24.0, 24.7, 26.7).
+      constexpr int JB = ROT ? D / 64 : 1;
 #pragma unroll
       for (int jb = 0; jb < NKS; jb += JB) {
         if (jb >= ngl) continue;  // warp-uniform
-        float2 ak[ROT ? JB : 1][ROT ? NKG / 2 : 1][2][2], at[ROT ? JB : 1][2];
+        float2 at[ROT ? JB : 1][2];
         if (ROT) {
 #pragma unroll
           for (int jj = 0; jj < JB; ++jj)
 #pragma unroll
-            for (int c = 0; c < 2; ++c) {
-              const int p = 8 * (jb + jj) + 4 * c + t4;
-              at[jj][c] = lds_f2(ks + TL_STAGE_BYTES + p * 8);
-#pragma unroll
-              for (int kp = 0; kp < NKG / 2; ++kp)
-#pragma unroll
-                for (int h2 = 0; h2 < 2; ++h2) ak[jj][kp][c][h2] = __ldg(P.rot_key + p * KT + warp * KB + (2 * kp + h2) * 8 + g);
-            }
+            for (int c = 0; c < 2; ++c) at[jj][c] = lds_f2(ks + TL_STAGE_BYTES + (8 * (jb + jj) + 4 * c + t4) * 8);
         }
 #pragma unroll
         for (int jj = 0; jj < JB; ++jj) {
@@ -722,9 +750,7 @@ atf_decode_tiles_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_co
             if (ROT) {
               // bf[2 * h2 + c] is pair 8j + 4c + t4 of key (2kp + h2) * 8 + g of the warp's part of the tile
 #pragma unroll
-              for (int c = 0; c < 2; ++c)
-#pragma unroll
-                for (int h2 = 0; h2 < 2; ++h2) bf[2 * h2 + c] = rotate_pair(bf[2 * h2 + c], at[jj][c], ak[jj][kp][c][h2]);
+              for (int c = 0; c < 2; ++c) rotate_pairs(bf[c], bf[2 + c], at[jj][c], kc[j][c][kp], ksi[j][c][kp]);
             }
 #pragma unroll
             for (int h2 = 0; h2 < 2; ++h2) {
@@ -732,8 +758,7 @@ atf_decode_tiles_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_co
               if (8 * j + t4 >= live) bf[2 * h2] = 0u;
               if (8 * j + 4 + t4 >= live) bf[2 * h2 + 1] = 0u;
             }
-            mma_bf16_16816(sc[2 * kp], qa[j][0], qa[j][1], bf[0], bf[1]);
-            mma_bf16_16816(sc[2 * kp + 1], qa[j][0], qa[j][1], bf[2], bf[3]);
+            mma_bf16_full(sc[kp], bf[0], bf[2], bf[1], bf[3], qa[j][0], qa[j][1]);
           }
         }
       }
@@ -743,53 +768,60 @@ atf_decode_tiles_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_co
           if (kb0 + kg * 8 + g < L) cnt += (unsigned long long)(H - r_lane[kg]);
       }
 
-      // ---- online softmax (log2 domain); this lane holds keys 2t, 2t+1 of every group of 8 keys for head g ----
-      float mx = -INFINITY;
+      // ---- online softmax (log2 domain); this lane holds keys g, g + 8 of every 16 for heads 2 t4 and 2 t4 + 1 ----
+      float mx[2] = {-INFINITY, -INFINITY};
       if (blk_fast) {
 #pragma unroll
-        for (int kg = 0; kg < NKG; ++kg)
+        for (int kp = 0; kp < NKG / 2; ++kp)
 #pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            sc[kg][e] *= kScaleLog2;
-            mx = fmaxf(mx, sc[kg][e]);
+          for (int e = 0; e < 4; ++e) {
+            sc[kp][e] *= kScaleLog2;
+            mx[e & 1] = fmaxf(mx[e & 1], sc[kp][e]);
           }
       } else {
 #pragma unroll
-        for (int kg = 0; kg < NKG; ++kg)
+        for (int kp = 0; kp < NKG / 2; ++kp)
 #pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            const int key = kb0 + kg * 8 + 2 * t4 + e;
-            sc[kg][e] = (key < L && L - 1 - key <= Wmax) ? sc[kg][e] * kScaleLog2 : -INFINITY;
-            mx = fmaxf(mx, sc[kg][e]);
+          for (int e = 0; e < 4; ++e) {
+            const int key = kb0 + kp * 16 + (e >> 1) * 8 + g;
+            sc[kp][e] = (key < L && L - 1 - key <= Wmax) ? sc[kp][e] * kScaleLog2 : -INFINITY;
+            mx[e & 1] = fmaxf(mx[e & 1], sc[kp][e]);
           }
       }
-      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-      float scale_o = 1.f;
+#pragma unroll
+      for (int off = 4; off < 32; off <<= 1) {
+        mx[0] = fmaxf(mx[0], __shfl_xor_sync(0xffffffffu, mx[0], off));
+        mx[1] = fmaxf(mx[1], __shfl_xor_sync(0xffffffffu, mx[1], off));
+      }
+      float scale_o[2] = {1.f, 1.f}, mref[2];
       bool moved = false;
-      if (mx > m_used + (m_used == -INFINITY ? 0.f : DEC_RESCALE_THRESHOLD)) {
-        scale_o = (m_used == -INFINITY) ? 0.f : ex2f(m_used - mx);
-        m_used = mx;
-        moved = true;
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        if (mx[i] > m_used[i] + (m_used[i] == -INFINITY ? 0.f : DEC_RESCALE_THRESHOLD)) {
+          scale_o[i] = (m_used[i] == -INFINITY) ? 0.f : ex2f(m_used[i] - mx[i]);
+          m_used[i] = mx[i];
+          moved = true;
+        }
+        mref[i] = (m_used[i] == -INFINITY) ? 0.f : m_used[i];
       }
       if (__any_sync(0xffffffffu, moved)) {
-        l_part *= scale_o;
+        l_part[0] *= scale_o[0];
+        l_part[1] *= scale_o[1];
 #pragma unroll
-        for (int nt = 0; nt < NNT; ++nt) {
-          oacc[nt][0] *= scale_o;
-          oacc[nt][1] *= scale_o;
-        }
+        for (int np = 0; np < NNT / 2; ++np)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) oacc[np][e] *= scale_o[e & 1];
       }
-      const float mref = (m_used == -INFINITY) ? 0.f : m_used;
-      uint32_t pa[NKG];
+      uint32_t pb[NKG];
 #pragma unroll
       for (int kg = 0; kg < NKG; ++kg) {
-        const float p0 = ex2f(sc[kg][0] - mref), p1 = ex2f(sc[kg][1] - mref);
-        l_part += p0 + p1;
-        pa[kg] = pack_bf16x2(p0, p1);
+        const float p0 = ex2f(sc[kg >> 1][2 * (kg & 1)] - mref[0]), p1 = ex2f(sc[kg >> 1][2 * (kg & 1) + 1] - mref[1]);
+        l_part[0] += p0;
+        l_part[1] += p1;
+        pb[kg] = movmatrix_trans(pack_bf16x2(p0, p1));  // key g, heads 2 t4 + {0, 1} -> head g, keys 2 t4 + {0, 1}
       }
 
-      // ---- O += P V (V tile in 128-byte-swizzled 64-column boxes) ----
+      // ---- O^T += V^T P^T (V tile in 128-byte-swizzled 64-column boxes) ----
 #pragma unroll
       for (int pk = 0; pk < NKG / 2; ++pk) {
 #pragma unroll
@@ -797,8 +829,7 @@ atf_decode_tiles_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_co
           const int chunk = 2 * np + (lm_i >> 1);  // 16-byte column chunk of the row, 0 .. D/8 - 1
           uint32_t bf[4];
           ldsm_x4_trans(vs + (chunk >> 3) * (KT * 128) + pk * 2048 + v_row_off + (((chunk & 7) ^ lm_r) << 4), bf);
-          mma_bf16_16816(oacc[2 * np], pa[2 * pk], pa[2 * pk + 1], bf[0], bf[1]);
-          mma_bf16_16816(oacc[2 * np + 1], pa[2 * pk], pa[2 * pk + 1], bf[2], bf[3]);
+          mma_bf16_full(oacc[np], bf[0], bf[2], bf[1], bf[3], pb[2 * pk], pb[2 * pk + 1]);
         }
       }
       __syncwarp();
@@ -807,24 +838,31 @@ atf_decode_tiles_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_co
   }
 
   // ---- merge the warps of the block (the ring is free once everybody is here) ----
-  l_part += __shfl_xor_sync(0xffffffffu, l_part, 1);
-  l_part += __shfl_xor_sync(0xffffffffu, l_part, 2);
+#pragma unroll
+  for (int off = 4; off < 32; off <<= 1) {
+    l_part[0] += __shfl_xor_sync(0xffffffffu, l_part[0], off);
+    l_part[1] += __shfl_xor_sync(0xffffffffu, l_part[1], off);
+  }
   if (fail_site) {
     atomicExch(P.status, 1u);
     atomicExch(P.status + 1, fail_site);
   }
   __syncthreads();
   float* sm = reinterpret_cast<float*>(sgen);  // [DEC_WARPS][G][PSTRIDE]
-  if (warp < DEC_WARPS && g < G) {
-    float* dst = sm + (warp * G + g) * PSTRIDE;
-    if (t4 == 0) {
-      dst[0] = m_used;
-      dst[1] = l_part;
-    }
+  if (warp < DEC_WARPS) {
 #pragma unroll
-    for (int nt = 0; nt < NNT; ++nt) {
-      dst[2 + nt * 8 + 2 * t4] = oacc[nt][0];
-      dst[2 + nt * 8 + 2 * t4 + 1] = oacc[nt][1];
+    for (int i = 0; i < 2; ++i) {
+      if (2 * t4 + i >= G) break;
+      float* dst = sm + (warp * G + 2 * t4 + i) * PSTRIDE;
+      if (g == 0) {
+        dst[0] = m_used[i];
+        dst[1] = l_part[i];
+      }
+#pragma unroll
+      for (int np = 0; np < NNT / 2; ++np) {
+        dst[2 + np * 16 + g] = oacc[np][i];
+        dst[2 + np * 16 + 8 + g] = oacc[np][2 + i];
+      }
     }
   }
   __syncthreads();
