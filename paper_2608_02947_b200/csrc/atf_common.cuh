@@ -43,6 +43,27 @@ AtfWorkspace atf_bound_workspace();
 // atf_check_status also reads (and clears) the status words registered here for the device
 void atf_register_status_words(int device, void* dev_ptr);
 
+#ifdef __CUDACC__
+// Launch that may overlap the end of the kernel before it in the stream (programmatic dependent launch): what the kernel does
+// in front of grid_dependency_wait() runs while that one drains, and the launch itself is off the critical path (two sequences
+// of 32768 keys, row cache, 24 heads: decode step 52.0 -> 49.4 us).  A kernel launched so waits before it reads or writes global
+// memory; the prefill's loads of Q in front of its wait are covered by the pre-pass, which lets it start behind its own wait.
+template <typename... KArgs, typename... Args>
+static inline cudaError_t atf_launch_overlapped(void (*kern)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t s, const Args&... args) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+#endif
+
 // Tiled TMA map of a [BH, N, D] bf16 tensor (heads head_rows rows apart): 64-column x box_rows boxes, 128-byte swizzle.
 atf_status atf_make_tile_map(CUtensorMap* m, const void* base, int64_t BH, int64_t N, int D, int64_t head_rows,
                              int box_rows);
@@ -72,6 +93,12 @@ __device__ __forceinline__ unsigned long long global_timer_ns() {
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
 }
+
+// ---- programmatic dependent launch ----
+// A kernel launched to overlap its predecessor in the stream waits here before it touches what that one wrote; the
+// predecessor lets it start (as soon as all its blocks have begun) with the other call.
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_dependency_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // ---- mbarrier ----
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {

@@ -199,6 +199,8 @@ atf_decode_kernel(const __grid_constant__ DecodeParams P, const __grid_constant_
   if (threadIdx.x < H) sW[threadIdx.x] = table.w[threadIdx.x];
   __syncthreads();
   const int Wmax = sW[H - 1];
+  grid_dependency_wait();
+  grid_dependency_launch();
 
   // A fragments of q for every K step: rows = heads of the group (rows >= G stay zero); K step j
   // contracts dims 16j..16j+15.
@@ -589,6 +591,8 @@ atf_decode_tiles_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_co
     tma_prefetch_desc(&tmV);
   }
   __syncthreads();
+  grid_dependency_wait();
+  grid_dependency_launch();
   const int Wmax = sW[H - 1];
   // the first tile that holds a key some pair reaches; tiles are dealt round-robin to the splits
   const int t_lo = max(0, L - 1 - Wmax) / KT;
@@ -946,7 +950,7 @@ atf_status launch_decode(const DecodeParams& P, const AtfTable& t, int B, int mo
     ATF_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));      \
     ATF_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,           \
                                         cudaSharedmemCarveoutMaxShared));                                \
-    kern<<<grid, DEC_THREADS, smem, s>>>(P, t);                                                     \
+    ATF_CUDA_CHECK(atf_launch_overlapped(kern, grid, DEC_THREADS, smem, s, P, t));                      \
   } while (0)
   if (mode == ATF_MODE_EXACT) {
     if (count) ATF_DEC_LAUNCH(ATF_MODE_EXACT, true); else ATF_DEC_LAUNCH(ATF_MODE_EXACT, false);
@@ -970,7 +974,7 @@ atf_status launch_decode_tiles(const CUtensorMap& tmV, const DecodeParams& P, co
     ATF_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));          \
     ATF_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,               \
                                         cudaSharedmemCarveoutMaxShared));                                    \
-    kern<<<grid, TL_THREADS, smem, s>>>(tmV, P, t);                                                           \
+    ATF_CUDA_CHECK(atf_launch_overlapped(kern, grid, TL_THREADS, smem, s, tmV, P, t));                      \
   } while (0)
   if (mode == ATF_MODE_EXACT) {
     if (count) ATF_TL_LAUNCH(ATF_MODE_EXACT, true); else ATF_TL_LAUNCH(ATF_MODE_EXACT, false);

@@ -31,6 +31,7 @@ atf_prefill_prep_kernel(const __grid_constant__ AtfTable table, int mode, int nd
                         const __nv_bfloat16* __restrict__ X, __nv_bfloat16* __restrict__ Y, int64_t rows, int D,
                         int64_t n_per_head, int64_t src_head_rows, __nv_bfloat16* __restrict__ Kg, int64_t kg_tiles,
                         int64_t kg_first_row) {
+  grid_dependency_wait();  // before the prefill kernel may start: it reads Q ahead of its own wait
   grid_dependency_launch();
   const int H = D / 2, per_row = D / 16;
   if ((int)blockIdx.x < sched_blocks) return atf_write_schedule(table, mode, H, ndt, sched);
@@ -139,9 +140,9 @@ atf_status atf_prefill_impl(const void* Q, const void* K, const void* V, void* O
     __nv_bfloat16* Kg = opts ? (__nv_bfloat16*)opts->kcache_groups : nullptr;
     const int64_t kt = 8192 / d;
     const int64_t kg_tiles = Kg ? (opts->kcache_capacity + kt - 1) / kt : 0;
-    atf_prefill_prep_kernel<<<(unsigned)blocks, ATF_PREP_THREADS, 0, s>>>(
-        t, mode, (int)((N + T - 1) / T), sb, sched, (const __nv_bfloat16*)K, Kp, rows_k, d, N, kv_head_rows, Kg, kg_tiles, N - Nq);
-    ATF_CUDA_CHECK(cudaGetLastError());
+    ATF_CUDA_CHECK(atf_launch_overlapped(
+        atf_prefill_prep_kernel, dim3((unsigned)blocks), ATF_PREP_THREADS, 0, s, t, mode, (int)((N + T - 1) / T), sb, sched, (const __nv_bfloat16*)K,
+        Kp, rows_k, d, N, kv_head_rows, Kg, kg_tiles, N - Nq));
   }
 
   CUtensorMap tk, tv;

@@ -31,10 +31,6 @@ constexpr int ATF_PREP_THREADS = 256;
 inline int atf_sched_blocks(int64_t N) { return (int)(((N + 127) / 128 + ATF_PREP_THREADS / 8 - 1) / (ATF_PREP_THREADS / 8)); }
 
 #ifdef __CUDACC__
-// A kernel launched to overlap its predecessor in the stream waits here before it touches what that one wrote; the
-// predecessor lets it start (as soon as all its blocks have begun) with the other call.
-__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_dependency_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 // A schedule word: an ordinary load that stays behind the wait.  The pre-pass may still be writing when the kernel that
 // reads starts, and the read-only path (__ldg) is defined only for what nothing writes while that kernel is resident.
 __device__ __forceinline__ uint32_t ld_sched(const uint32_t* p) {

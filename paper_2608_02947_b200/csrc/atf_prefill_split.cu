@@ -30,6 +30,7 @@ atf_split_prep_kernel(const __grid_constant__ AtfTable table, int mode, int ndt,
                       const float* __restrict__ Q, const float* __restrict__ K, __nv_bfloat16* __restrict__ Qhi,
                       __nv_bfloat16* __restrict__ Qlo, __nv_bfloat16* __restrict__ Khi, __nv_bfloat16* __restrict__ Klo,
                       int64_t rows_q, int64_t rows_k, int D) {
+  grid_dependency_wait();
   grid_dependency_launch();
   const int H = D / 2, per_row = D / 16;
   if ((int)blockIdx.x < sched_blocks) return atf_write_schedule(table, mode, H, ndt, sched);
@@ -119,10 +120,9 @@ extern "C" atf_status atf_prefill_split_chunk(const float* Q, const float* K, co
     const int sb = atf_sched_blocks(N);
     const int64_t blocks = sb + ((rows_q + rows_k) * (d / 16) + ATF_PREP_THREADS - 1) / ATF_PREP_THREADS;
     if (blocks > 0x7FFFFFFF) return atf_fail(ATF_ERR_UNSUPPORTED, "atf_prefill_split: problem too large for the repack grid");
-    atf_split_prep_kernel<<<(unsigned)blocks, ATF_PREP_THREADS, 0, s>>>(t, mode, (int)((N + T - 1) / T), sb,
+    ATF_CUDA_CHECK(atf_launch_overlapped(atf_split_prep_kernel, dim3((unsigned)blocks), ATF_PREP_THREADS, 0, s, t, mode, (int)((N + T - 1) / T), sb,
                                                                         (uint32_t*)(base + ATF_WS_HEADER), Q, K, Qhi, Qlo, Khi,
-                                                                        Klo, rows_q, rows_k, d);
-    ATF_CUDA_CHECK(cudaGetLastError());
+                                                                        Klo, rows_q, rows_k, d));
   }
   CUtensorMap tqh, tql, tkh, tkl, tv;
   if ((st = atf_make_tile_map(&tqh, Qhi, (int64_t)B * Hq, Nq, d, Nq, T)) != ATF_OK) return st;

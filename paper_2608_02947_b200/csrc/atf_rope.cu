@@ -56,6 +56,7 @@ __global__ void __launch_bounds__(ROPE_THREADS) atf_rope_kernel(T* __restrict__ 
   constexpr int SEGS = ROPE_THREADS / HL;               // (row, segment) pairs of the block
   constexpr int ROWS = SEGS / CHUNKS;
   const int64_t row0 = (int64_t)blockIdx.x * ROWS;
+  grid_dependency_launch();
   const int sg = threadIdx.x % SEGS, c = sg % CHUNKS;
   const int64_t n = row0 + sg / CHUNKS;
   double cs[8], sn[8];
@@ -92,6 +93,7 @@ __global__ void __launch_bounds__(ROPE_THREADS) atf_rope_kernel(T* __restrict__ 
     store8(row, olo);
     store8(row + H, ohi);
   };
+  grid_dependency_wait();  // the angles need nothing of the kernel before
   const int64_t head = N * D;
   const int lane = threadIdx.x / SEGS;
   const int first = SPREAD ? (int)blockIdx.y * HL + lane : lane, step = SPREAD ? HL * (int)gridDim.y : HL;
@@ -133,7 +135,7 @@ __global__ void __launch_bounds__(ROPE_THREADS) atf_rope_kernel(T* __restrict__ 
 // the next one is on its way (192 heads x 2048 96 -> 69 us, 24 x 32768 200 -> 132, 24 x 131072 603 -> 504); smaller
 // data is slower so (24 x 8192 31.6 -> 33.0), and so is bf16 (24 x 131072 272 -> 306).
 template <int D, typename T>
-static void launch_rope(T* X, int BH, int64_t N, int64_t pos0, const RopeTheta& th, cudaStream_t s) {
+static cudaError_t launch_rope(T* X, int BH, int64_t N, int64_t pos0, const RopeTheta& th, cudaStream_t s) {
   constexpr bool F32 = sizeof(T) == 4;
   const auto blocks = [&](int lanes) { return (N + ROPE_THREADS / lanes / (D / 16) - 1) / (ROPE_THREADS / lanes / (D / 16)); };
   int hl = 1;
@@ -144,19 +146,14 @@ static void launch_rope(T* X, int BH, int64_t N, int64_t pos0, const RopeTheta& 
   const unsigned g = (unsigned)blocks(hl), want = (F32 ? 12 : 3) * 148;
   if (!pre && hl == 8 && BH > 8 && g < want) {
     const unsigned gy = std::min(((unsigned)BH + 7) / 8, (want + g - 1) / g);
-    atf_rope_kernel<D, 8, T, true><<<dim3(g, gy), ROPE_THREADS, 0, s>>>(X, BH, N, pos0, th);
-    return;
+    return atf_launch_overlapped(atf_rope_kernel<D, 8, T, true>, dim3(g, gy), ROPE_THREADS, 0, s, X, BH, N, pos0, th);
   }
-#define ATF_ROPE_LAUNCH(HL_)                                                                        \
-  do {                                                                                              \
-    if (pre) atf_rope_kernel<D, HL_, T, false, F32><<<g, ROPE_THREADS, 0, s>>>(X, BH, N, pos0, th);  \
-    else atf_rope_kernel<D, HL_, T><<<g, ROPE_THREADS, 0, s>>>(X, BH, N, pos0, th);                 \
-  } while (0)
-  if (hl == 1) ATF_ROPE_LAUNCH(1);
-  else if (hl == 2) ATF_ROPE_LAUNCH(2);
-  else if (hl == 4) ATF_ROPE_LAUNCH(4);
-  else ATF_ROPE_LAUNCH(8);
-#undef ATF_ROPE_LAUNCH
+  void (*kern)(T*, int, int64_t, int64_t, RopeTheta);
+  if (hl == 1) kern = pre ? atf_rope_kernel<D, 1, T, false, F32> : atf_rope_kernel<D, 1, T>;
+  else if (hl == 2) kern = pre ? atf_rope_kernel<D, 2, T, false, F32> : atf_rope_kernel<D, 2, T>;
+  else if (hl == 4) kern = pre ? atf_rope_kernel<D, 4, T, false, F32> : atf_rope_kernel<D, 4, T>;
+  else kern = pre ? atf_rope_kernel<D, 8, T, false, F32> : atf_rope_kernel<D, 8, T>;
+  return atf_launch_overlapped(kern, dim3(g), ROPE_THREADS, 0, s, X, BH, N, pos0, th);
 }
 
 template <typename T>
@@ -169,11 +166,8 @@ static atf_status rope(const char* who, T* X, int B, int H, int64_t N, int d, co
   for (int r = 0; r < d / 2; ++r) th.t[r] = theta[r];
   for (int r = d / 2; r < ATF_MAX_PAIRS; ++r) th.t[r] = 0.0;
   if ((N * (d / 16) + 255) / 256 > 0x7FFFFFFF) return atf_fail(ATF_ERR_UNSUPPORTED, "%s: N too large", who);
-  if (d == 64)
-    launch_rope<64>(X, B * H, N, pos0, th, (cudaStream_t)stream);
-  else
-    launch_rope<128>(X, B * H, N, pos0, th, (cudaStream_t)stream);
-  ATF_CUDA_CHECK(cudaGetLastError());
+  ATF_CUDA_CHECK(d == 64 ? launch_rope<64>(X, B * H, N, pos0, th, (cudaStream_t)stream)
+                         : launch_rope<128>(X, B * H, N, pos0, th, (cudaStream_t)stream));
   return ATF_OK;
 }
 

@@ -1,0 +1,85 @@
+"""Kernels launched to overlap the one before them in the stream: chains in which every call reads what the call before wrote give
+what they give with a synchronisation between any two."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("d,L", [(128, 3000), (64, 200)])
+def test_chain_of_dependent_calls(d, L):
+    import paper_2608_02947_b200 as atf
+    B, Hq, Hkv = 2, 6, 2
+    g = torch.Generator(device="cuda").manual_seed(L)
+    W, theta = atf.atf_window_table(5e5, d, 2.0, L)
+    table = atf.WindowTable(W)
+    K, V = [torch.randn((B, Hkv, L, d), generator=g, device="cuda").to(torch.bfloat16) for _ in range(2)]
+    q0 = torch.randn((B, Hq, d), generator=g, device="cuda").to(torch.bfloat16)
+    Kg = atf.new_kcache_groups(B, Hkv, L, d, "cuda")
+    q, k, Qn = torch.empty_like(q0), torch.empty_like(K), torch.empty((B, Hq, L, d), dtype=torch.bfloat16, device="cuda")
+    O = torch.empty_like(Qn)
+
+    def chain(sync):
+        out = []
+        wait = torch.cuda.synchronize if sync else (lambda: None)
+        q.copy_(q0)
+        for i in range(6):
+            k.copy_(K)
+            for X, pos in ((q[:, :, None], L - 1 + i), (k, i)):
+                wait()
+                atf.atf_rope(X, theta, pos0=pos)  # in place, read by the next call
+            wait()
+            a = atf.atf_decode(q, k, V, table=table, O=torch.empty_like(q))
+            wait()
+            atf.atf_decode(a, k, V, table=table, O=q)  # the query of the next calls
+            wait()
+            Qn.copy_(q[:, :, None].expand_as(Qn))
+            atf.atf_rope(Qn, theta)
+            wait()
+            _, lse = atf.atf_prefill(Qn, k, V, table=table, O=O, kcache_groups=Kg)
+            wait()
+            b = atf.atf_decode(O[:, :, -1].contiguous(), Kg, V, table=table)
+            wait()
+            atf.atf_decode(b, Kg, V, table=table, O=q)
+            out += [a, b, lse, q.clone()]
+        torch.cuda.synchronize()
+        return out
+
+    want = chain(True)
+    for _ in range(10):
+        for x, y in zip(want, chain(False)):
+            assert torch.equal(x, y)
+
+
+def test_captured_chain():
+    import paper_2608_02947_b200 as atf
+    B, Hq, Hkv, d, L = 1, 6, 2, 128, 700
+    g = torch.Generator(device="cuda").manual_seed(L)
+    W, theta = atf.atf_window_table(5e5, d, 2.0, L)
+    table = atf.WindowTable(W)
+    K, V = [torch.randn((B, Hkv, L, d), generator=g, device="cuda").to(torch.bfloat16) for _ in range(2)]
+    q0 = torch.randn((B, Hq, d), generator=g, device="cuda").to(torch.bfloat16)
+    q = q0.clone()
+
+    def steps(wait):
+        got = []
+        for i in range(4):
+            atf.atf_rope(q[:, :, None], theta, pos0=L + i)
+            wait()
+            got.append(atf.atf_decode(q, K, V, table=table))
+            wait()
+            atf.atf_decode(got[-1], K, V, table=table, O=q)
+            wait()
+        return got
+
+    want = steps(torch.cuda.synchronize)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        got = steps(lambda: None)
+    for _ in range(3):
+        q.copy_(q0)
+        graph.replay()
+        torch.cuda.synchronize()
+        for a, b in zip(want, got):
+            assert torch.equal(a, b)
