@@ -11,6 +11,11 @@
 //               tensor memory, V through the MN-major descriptor);
 //   warps 4-7   softmax group 0: keys 0..63 of every tile, one query row per thread;
 //   warps 8-11  softmax group 1: keys 64..127 of the same rows.
+// TURNS (coarse mode; which calls: launch_pipe): behind the diagonal tile the groups take whole tiles in turn instead, so that one
+// group's waits and tensor-memory round trips fall into the other's exponentials, and a tile has one of each where it had two.
+// The sums of a tile's two key halves then go through shared memory to warp 2, which adds them in the order of the tiles, as the
+// two threads of a row do otherwise; at d = 128 the second copy of the exchange area takes the third K stage's place (a second
+// copy is worth it: with one, 8192 rows 439 us, with two and three K but two V stages 461, so 410).
 // The softmax warps also bring Q in (half a row each, again per pass, see below): they read the caller's rows and
 // store them to shared memory in the column order of atf_prefill.cu.  A row of Q is read by one CTA only, so a pre-pass
 // that reorders it would move it twice more (8192 rows of 24 heads: 22 us of 700).  The split-precision mode keeps such
@@ -63,12 +68,12 @@ static_assert(128 * 56 + 256 * 224 <= PP_THREADS * 168, "setmaxnreg budget excee
 // Q parts, a K stage is a hi tile followed by a lo tile, and the rings shrink to two K stages and one V stage.
 // QCOPY (exact mode, bf16 inputs): a second copy of Q that stays whole, for the per-cell finish; at d = 128 it takes the
 // place of the third K stage.
-template <int D, bool SPLIT, bool QCOPY>
+template <int D, bool SPLIT, bool QCOPY, bool TURNS>
 struct PipeSmem {
   static constexpr int NB = D / 64;
   static constexpr int TILE = NB * BLK_BYTES;
   static constexpr int QN = SPLIT ? 2 : 1;       // operand parts: hi, lo
-  static constexpr int KS = SPLIT || (QCOPY && D == 128) ? 2 : 3;  // ring depths
+  static constexpr int KS = SPLIT || ((QCOPY || TURNS) && D == 128) ? 2 : 3;  // ring depths
   static constexpr int VS = SPLIT ? 1 : 3;
   static constexpr int KSTAGE = QN * TILE;
   static constexpr int Q_OFF = 0;                // hi part, then lo part
@@ -76,8 +81,8 @@ struct PipeSmem {
   static constexpr int V_OFF = K_OFF + KS * KSTAGE;
   static constexpr int QC_OFF = V_OFF + VS * TILE;
   static constexpr int BAR_OFF = QC_OFF + (QCOPY ? TILE : 0);
-  static constexpr int X_OFF = BAR_OFF + 256;  // exchange area of the two softmax groups: [2][128] floats
-  static constexpr int TOTAL = X_OFF + 1024;
+  static constexpr int X_OFF = BAR_OFF + 256;  // exchange area of the two softmax groups: [2][128] floats, in turns two of them
+  static constexpr int TOTAL = X_OFF + (TURNS ? 2048 : 1024);
   static constexpr int DYN_BYTES = TOTAL + 1024;  // slack for 1024-byte alignment
 };
 enum { B_QFULL = 0, B_KFULL = 1, B_KEMPTY = 4, B_VFULL = 7, B_VEMPTY = 10, B_SFULL = 13, B_SREAD = 15, B_PFULL = 17,
@@ -169,14 +174,14 @@ __device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, vol
   }
 }
 
-template <int D, int MODE, bool COUNT, bool SPLIT>
+template <int D, int MODE, bool COUNT, bool SPLIT, bool TURNS>
 __global__ void __launch_bounds__(PP_THREADS, 1)
 atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmQlo,
                         const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmKlo,
                         const __grid_constant__ CUtensorMap tmV, const __grid_constant__ AtfPipeParams P,
                         const __grid_constant__ AtfTable table) {
   constexpr bool QCOPY = MODE == ATF_MODE_EXACT && !SPLIT;
-  using SM = PipeSmem<D, SPLIT, QCOPY>;
+  using SM = PipeSmem<D, SPLIT, QCOPY, TURNS>;
   constexpr int KS = SM::KS, VS = SM::VS;
   constexpr int POLY = SPLIT ? 0 : ATF_PIPE_POLY_OF_4;
   constexpr int H = D / 2;
@@ -295,8 +300,10 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             tma_load_3d(sV + vs * SM::TILE + kb * BLK_BYTES, &tmV, bar(B_VFULL + vs), kb * 64, (it - t) * T, bhk);
           return true;
         };
-        if (SPLIT) {
-          // one V stage: V(t) has to wait for O += P(t - 1) V, so K(t + 1) goes first
+        if (SPLIT || TURNS || D == 128) {
+          // S runs ahead of O += P V: K(t + 1) in front of V(t), which may have to wait for a product (24 heads x 8192 rows of 128,
+          // coarse: 423 -> 410 us in turns; exact, a layer step: 650 -> 644; 14 heads x 32768 of 64, exact, the other way: 2843
+          // against 2822)
           bool pok = nt == 0 || load_k(0);
           for (int t = 0; t < nt && pok; ++t) pok = (t + 1 >= nt || load_k(t + 1)) && load_v(t);
           if (!pok) fail_site = 10;
@@ -349,10 +356,12 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
     for (int pass = 0; pass < 2; ++pass) {
       const int g0 = pass * nt;
-      if (lane == 0) {
-        bool iok = true;
-        for (int t = 0; t < nt && iok; ++t) {
-          const int g = g0 + t, sb = g & 1, vs = g % VS;
+      const bool sums = TURNS && pass == 0;  // the whole warp walks the steps, else lane 0 alone
+      float sum[2][4] = {};                  // rows 4 lane .. 4 lane + 3, keys 0..63 and 64..127 of the tiles so far
+      bool iok = true;
+      for (int t = 0; t < nt && iok && (sums || lane == 0); ++t) {
+        const int g = g0 + t, sb = g & 1, vs = g % VS;
+        if (lane == 0) {
           const uint64_t dV = make_smem_desc_sw128(sV + vs * SM::TILE, BLK_BYTES, 1024);
           const uint32_t tO = tmem_base + 2 * T, tP = tmem_base + 3 * T + sb * 64;
           iok = wait_or_abort(bar(B_VFULL + vs), (g / VS) & 1, abortp);
@@ -365,11 +374,32 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
               tc_mma_ts(tO, tP + 32 * h + 8 * i, dV + (uint64_t)(512 * h + 128 * i), IDESC_PV,
                         (t > 0 || h > 0 || i > 0) ? 1u : 0u);
           }
-          if (!iok) { fail_site = 22; break; }
+          if (!iok) fail_site = 22;
+        }
+        if (sums) {
+          // the tile's sums, added in the order of the tiles
+          iok = __shfl_sync(0xffffffffu, (int)iok, 0);
+          if (!iok) break;
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            float v[4];
+            lds_f4(smem_base + SM::X_OFF + ((2 * sb + h) * 128 + 4 * lane) * 4, v);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) sum[h][i] += v[i];
+          }
+          __syncwarp();
+        }
+        if (lane == 0 && iok) {
           tc_commit(bar(B_VEMPTY + vs));
           tc_commit(bar(B_PVDONE + sb));
         }
-        if (iok) tc_commit(bar(B_OFULL));
+      }
+      if (lane == 0 && iok) tc_commit(bar(B_OFULL));
+      if (sums) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) xch[h * 128 + 4 * lane + i] = sum[h][i];
       }
       if (!another_pass(pass)) break;
     }
@@ -394,7 +424,7 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     float m_used = -INFINITY, l_run = 0.f;
     unsigned long long cnt = 0;
     uint32_t xphase = 0;
-    bool ok = true;
+    bool ok = true, redone = false;
     // all eight softmax warps meet (bounded): what each wrote to the exchange area before is visible after
     auto softmax_sync = [&]() {
       __syncwarp();
@@ -421,6 +451,7 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     for (int pass = 0; pass < 2; ++pass) {
       const int g0 = pass * nt;
       const bool safe = pass == 1;
+      redone = safe;
       uint32_t qw[QW];
       if constexpr (!SPLIT) load_q(qw);
       if (pass == 0) grid_dependency_wait();
@@ -475,9 +506,51 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       }
       int t = 0;
       while (t < nt && ok) {
+        if constexpr (TURNS) {
+          // ---- In turns: behind the diagonal tile group h takes the steps g with g % 2 == h, all 128 keys of its rows. ----
+          if (t > 0 && !safe) {
+            const float neg_m = -m_used * kScaleLog2;
+            const uint32_t tS = tmem_base + h * T + lane_off, tP = tmem_base + 3 * T + h * 64 + lane_off;
+            for (t += (g0 + t + h) & 1; t < nt; t += 2) {
+              const int g = g0 + t;
+              if (!wait_or_abort(bar(B_SFULL + h), (g >> 1) & 1, abortp)) { ok = false; fail_site = 31; break; }
+              tc_fence_after();
+              float sa[64], sb[64];
+              tc_ld32(tS, reinterpret_cast<uint32_t*>(sa));
+              tc_ld32(tS + 32, reinterpret_cast<uint32_t*>(sa) + 32);
+              tc_wait_ld();
+              tc_ld32(tS + 64, reinterpret_cast<uint32_t*>(sb));  // on its way behind the first half's exponentials
+              tc_ld32(tS + 96, reinterpret_cast<uint32_t*>(sb) + 32);
+              uint32_t pk[32];
+              const float la = exp_half<POLY>(sa, kScaleLog2, neg_m, pk);
+              // the product that read the previous contents of this P buffer must be complete
+              if (g >= 2 && !wait_or_abort(bar(B_PVDONE + h), ((g - 2) >> 1) & 1, abortp)) { ok = false; fail_site = 35; break; }
+              tc_fence_after();
+              tc_st32(tP, pk);
+              tc_wait_ld_pin64(sb);
+              tc_wait_st();
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) {
+                mbar_arrive_n(bar(B_SREAD + h), 2);  // for the other group's warp too
+                mbar_arrive(bar(B_PFULL + 2 * h));
+              }
+              const float lb = exp_half<POLY>(sb, kScaleLog2, neg_m, pk);
+              tc_st32(tP + 32, pk);
+              overflow |= !(la < STALE_REF_GUARD) || !(lb < STALE_REF_GUARD);
+              xch[h * 256 + row] = la;  // PVDONE above: warp 2 has taken what was there
+              xch[h * 256 + 128 + row] = lb;
+              tc_wait_st();
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(bar(B_PFULL + 2 * h + 1));
+            }
+            break;
+          }
+        }
         // ---- plain steps: no mask, no per-cell finish, reference from the diagonal tile.  A loop of its own,
         //      kept small so that it stays in the instruction cache; everything else takes the general step. ----
-        for (; t < nt && !safe && t > 0; ++t) {
+        for (; !TURNS && t < nt && !safe && t > 0; ++t) {
           const int g = g0 + t, sb = g & 1, ks = g % KS;
           const PipeWord E(e_cur);
           if (!E.plain) break;
@@ -717,6 +790,7 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         if (g >= 2 && !wait_or_abort(bar(B_PVDONE + sb), ((g - 2) >> 1) & 1, abortp)) { ok = false; fail_site = 35; break; }
         tc_st32(tP, pk);
         l_run = l_run * scale_o + lsum;
+        if (TURNS && !safe) xch[h * 128 + row] = lsum;  // the diagonal tile's
         tc_wait_st();
         tc_fence_before();
         __syncwarp();
@@ -729,10 +803,12 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       if (!safe && overflow && row_ok) s_redo = 1;
       if (!another_pass(pass)) break;
     }
-    // ---- both halves of the row sum, then the output ----
-    xch[h * 128 + row] = l_run;
-    if (ok && !softmax_sync()) { ok = false; fail_site = 37; }
-    const float l_tot = l_run + xch[(h ^ 1) * 128 + row];
+    // ---- both halves of the row sum (after a fast pass in turns warp 2 has left them there), then the output ----
+    if (!TURNS || redone) {
+      xch[h * 128 + row] = l_run;
+      if (ok && !softmax_sync()) { ok = false; fail_site = 37; }
+    }
+    const float l_tot = xch[h * 128 + row] + xch[(h ^ 1) * 128 + row];
     if (ok && nt > 0) {
       tc_fence_after();
       const float inv = 1.f / l_tot;
@@ -788,18 +864,27 @@ atf_status launch_pipe(const CUtensorMap& tq, const CUtensorMap& tql, const CUte
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
   cfg.blockDim = dim3(PP_THREADS);
-#define ATF_PP_LAUNCH(MODE_, COUNT_)                                                                   \
+#define ATF_PP_LAUNCH(MODE_, COUNT_, TURNS_)                                                          \
   do {                                                                                                 \
-    auto kern = atf_prefill_pipe_kernel<D, MODE_, COUNT_, SPLIT>;                                      \
-    const int smem = PipeSmem<D, SPLIT, MODE_ == ATF_MODE_EXACT && !SPLIT>::DYN_BYTES;                 \
+    auto kern = atf_prefill_pipe_kernel<D, MODE_, COUNT_, SPLIT, TURNS_>;                              \
+    const int smem = PipeSmem<D, SPLIT, MODE_ == ATF_MODE_EXACT && !SPLIT, TURNS_>::DYN_BYTES;                 \
     ATF_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));     \
     cfg.dynamicSmemBytes = smem;                                                                       \
     ATF_CUDA_CHECK(cudaLaunchKernelEx(&cfg, kern, tq, tql, tk, tkl, tv, P, t));                        \
   } while (0)
+  // In turns or in step: the results are the same, bit for bit.  In turns pays where the softmax holds the pace and no warp has
+  // cells to finish (us, in step -> in turns: coarse, 24 heads of 128, 8192 rows 446 -> 410, 32768 5780 -> 5210, 4000 of 61003
+  // 2650 -> 2415; 14 heads of 64, 32768 rows, coarse 2636 -> 2400, full 2520 -> 2290).  Full attention at d = 128 and the split-
+  // precision form are bound by the tensor pipe (8192 rows, full 432 -> 449); exact mode's finish is slower by one warp for all
+  // 128 keys (8192 rows 596 -> 690), and a kernel with both forms of it slower in either; calls that count terms stay in step.
   if (mode == ATF_MODE_EXACT) {
-    if (count) ATF_PP_LAUNCH(ATF_MODE_EXACT, true); else ATF_PP_LAUNCH(ATF_MODE_EXACT, false);
+    if (count) ATF_PP_LAUNCH(ATF_MODE_EXACT, true, false); else ATF_PP_LAUNCH(ATF_MODE_EXACT, false, false);
+  } else if (count) {
+    ATF_PP_LAUNCH(ATF_MODE_COARSE, true, false);
+  } else if (!SPLIT && (D == 64 || t.w[0] < P.N - 1)) {
+    ATF_PP_LAUNCH(ATF_MODE_COARSE, false, !SPLIT);
   } else {
-    if (count) ATF_PP_LAUNCH(ATF_MODE_COARSE, true); else ATF_PP_LAUNCH(ATF_MODE_COARSE, false);
+    ATF_PP_LAUNCH(ATF_MODE_COARSE, false, false);
   }
 #undef ATF_PP_LAUNCH
   ATF_CUDA_CHECK(cudaGetLastError());
