@@ -28,13 +28,14 @@ constexpr int T = 128;  // query rows per tile and key columns per tile
 // rows from kg_first_row on.
 __global__ void __launch_bounds__(ATF_PREP_THREADS)
 atf_prefill_prep_kernel(const __grid_constant__ AtfTable table, int mode, int ndt, int sched_blocks, uint32_t* __restrict__ sched,
+                        int cuts, unsigned int* __restrict__ flags,
                         const __nv_bfloat16* __restrict__ X, __nv_bfloat16* __restrict__ Y, int64_t rows, int D,
                         int64_t n_per_head, int64_t src_head_rows, __nv_bfloat16* __restrict__ Kg, int64_t kg_tiles,
                         int64_t kg_first_row) {
   grid_dependency_wait();  // before the prefill kernel may start: it reads Q ahead of its own wait
   grid_dependency_launch();
   const int H = D / 2, per_row = D / 16;
-  if ((int)blockIdx.x < sched_blocks) return atf_write_schedule(table, mode, H, ndt, sched);
+  if ((int)blockIdx.x < sched_blocks) return atf_write_schedule(table, mode, H, ndt, sched, cuts, flags);
   const int64_t gid = (int64_t)(blockIdx.x - sched_blocks) * ATF_PREP_THREADS + threadIdx.x;
   if (gid >= rows * per_row) return;
   const int64_t row = gid / per_row;
@@ -130,6 +131,11 @@ atf_status atf_prefill_impl(const void* Q, const void* K, const void* V, void* O
   uint32_t* sched = (uint32_t*)(base + ATF_WS_HEADER);
   __nv_bfloat16* Kp = (__nv_bfloat16*)(base + ATF_WS_HEADER + sched_bytes(N));
   cudaStream_t s = (cudaStream_t)stream;
+  // The state of cut tiles lies where the reordered Q that `need` counts once was; a call that counts terms does not cut.
+  const size_t used = ATF_WS_HEADER + sched_bytes(N) + repack_bytes(B, Hkv, N, d);
+  const int cuts = opts && opts->kept_terms ? 0 : atf_prefill_cuts(N, Nq, (int64_t)B * Hq, t.w[d / 2 - 1], d, ws.bytes - used);
+  float* state = (float*)(base + used);
+  unsigned int* flags = (unsigned int*)(state + atf_cut_floats(d));
 
   {
     const int64_t rows_q = (int64_t)B * Hq * Nq, rows_k = (int64_t)B * Hkv * N;
@@ -141,7 +147,7 @@ atf_status atf_prefill_impl(const void* Q, const void* K, const void* V, void* O
     const int64_t kt = 8192 / d;
     const int64_t kg_tiles = Kg ? (opts->kcache_capacity + kt - 1) / kt : 0;
     ATF_CUDA_CHECK(atf_launch_overlapped(
-        atf_prefill_prep_kernel, dim3((unsigned)blocks), ATF_PREP_THREADS, 0, s, t, mode, (int)((N + T - 1) / T), sb, sched, (const __nv_bfloat16*)K,
+        atf_prefill_prep_kernel, dim3((unsigned)blocks), ATF_PREP_THREADS, 0, s, t, mode, (int)((N + T - 1) / T), sb, sched, cuts, flags, (const __nv_bfloat16*)K,
         Kp, rows_k, d, N, kv_head_rows, Kg, kg_tiles, N - Nq));
   }
 
@@ -155,6 +161,9 @@ atf_status atf_prefill_impl(const void* Q, const void* K, const void* V, void* O
   P.Qhi = P.Qlo = nullptr;
   P.O = (__nv_bfloat16*)O;
   P.LSE = LSE;
+  P.cuts = cuts;
+  P.flags = flags;
+  P.state = state;
   P.kept = opts ? (unsigned long long*)opts->kept_terms : nullptr;
   P.status = (unsigned int*)base;
   P.Hq = Hq;

@@ -174,7 +174,7 @@ __device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, vol
   }
 }
 
-template <int D, int MODE, bool COUNT, bool SPLIT, bool TURNS>
+template <int D, int MODE, bool COUNT, bool SPLIT, bool TURNS, bool CUT>
 __global__ void __launch_bounds__(PP_THREADS, 1)
 atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmQlo,
                         const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmKlo,
@@ -202,19 +202,36 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   __shared__ int sW[ATF_MAX_PAIRS];
   __shared__ int s_abort;
   __shared__ int s_redo;
+  __shared__ volatile int s_part[CUT ? 2 : 1];  // CUT: first step of the block in the fast pass; whether it ends at the cut
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int ntq = (P.N + T - 1) / T;
-  const int it = ntq - 1 - (int)blockIdx.x;  // longest rows first; the grid stops at the tile holding row n0
   const int n0 = P.N - P.Nq;
-  const int hq = blockIdx.y, b = blockIdx.z;
-  const int bhq = b * P.Hq + hq;
+  // Blocks start in the order of their index: the tiles of a group of heads, longest rows first.  CUT: the first P.cuts tiles
+  // are worked on by two blocks (atf_prefill_cuts).
+  const int ntq = (P.N + T - 1) / T;
+  const bool first = CUT && (int)blockIdx.x < P.cuts, second = CUT && (int)blockIdx.x >= P.jobs;
+  const int job = second ? (int)blockIdx.x - P.jobs : (int)blockIdx.x;
+  const int head0 = (int)blockIdx.y * P.group, heads = min(P.group, P.heads - head0);
+  const int it = ntq - 1 - job / heads;
+  if (it < n0 / T) return;  // the last group may have fewer heads
+  const int bhq = head0 + job % heads;
+  const int b = bhq / P.Hq, hq = bhq - b * P.Hq;
   const int bhk = b * P.Hkv + hq / (P.Hq / P.Hkv);
+  const int Wmax = table.w[H - 1];
+  const int dlim = (Wmax + T - 1) / T + 1;  // first tile distance no pair reaches
+  const int nt = min(it + 1, dlim);         // key tiles it, it - 1, ... walked outwards from the diagonal
+  const int cut = first || second ? (int)((long long)nt * (2 * job + 1) / (2 * P.cuts)) : 0;  // steps of the first block
+  if (first && cut == 0) return;
+  const int t_end = first ? cut : nt;
 
   if (tid < H) sW[tid] = table.w[tid];
   if (tid == 0) {
     s_abort = 0;
     s_redo = 0;
+    if (CUT) {
+      s_part[0] = second ? cut : 0;
+      s_part[CUT ? 1 : 0] = first;
+    }
     mbar_init(bar(B_QFULL), SPLIT ? 1 : 8);
     mbar_init(bar(B_OFULL), 1);
     mbar_init(bar(B_XCH), 8);
@@ -251,18 +268,39 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  const int Wmax = sW[H - 1];
-  const int dlim = (Wmax + T - 1) / T + 1;  // first tile distance no pair reaches
-  const int nt = min(it + 1, dlim);         // key tiles it, it - 1, ... walked outwards from the diagonal
   volatile int* abortp = &s_abort;
   unsigned int fail_site = 0;
+
+  // A cut tile's state: O (fp32, [D / 4][128 rows][4]), the sums of the two key halves, the rows' reference; and a flag (1: there,
+  // 2: a sum has overflowed, the whole tile takes the safe form).
+  auto cut_state = [&]() {
+    const int j = (int)blockIdx.x < P.cuts ? (int)blockIdx.x : (int)blockIdx.x - P.jobs;
+    return P.state + (int64_t)j * (T * (D + 3));
+  };
+  if (CUT && second && cut > 0) {
+    if (tid == 0) {
+      grid_dependency_wait();
+      const unsigned long long w0 = global_timer_ns();
+      unsigned int f;
+      while ((f = ld_acquire(P.flags + ((int)blockIdx.x - P.jobs))) == 0u && global_timer_ns() - w0 <= ATF_WAIT_LIMIT_NS) __nanosleep(200);
+      if (f == 0u) {
+        s_abort = 1;
+        fail_site = 40;
+      }
+      if (f == 2u) {
+        s_redo = 1;
+        s_part[0] = nt;  // no step of the fast pass
+      }
+    }
+    __syncthreads();
+  }
 
   // Every role runs the tile once and, if a softmax thread raised s_redo, once more in the safe form.  The
   // passes end at a CTA-wide barrier (the same barrier from every role's branch); barrier phases of the
   // pipeline run on across the passes (g = steps since the start of the kernel).
   auto another_pass = [&](int pass) {
     asm volatile("bar.sync 0;" ::: "memory");
-    return pass == 0 && *reinterpret_cast<volatile int*>(&s_redo) != 0;
+    return pass == 0 && !(CUT && s_part[CUT ? 1 : 0]) && *reinterpret_cast<volatile int*>(&s_redo) != 0;
   };
 
   if (warp == 0) {
@@ -270,7 +308,7 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
     grid_dependency_wait();
     for (int pass = 0; pass < 2; ++pass) {
-      const int g0 = pass * nt;
+      const int tb = CUT && !pass ? s_part[0] : 0, g0 = (pass ? t_end - (CUT ? s_part[0] : 0) : 0) - tb;  // g = g0 + t: steps of this block so far
       if (lane == 0) {
         if (SPLIT) {
           mbar_expect_tx(bar(B_QFULL), SM::QN * SM::TILE);
@@ -304,11 +342,11 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
           // S runs ahead of O += P V: K(t + 1) in front of V(t), which may have to wait for a product (24 heads x 8192 rows of 128,
           // coarse: 423 -> 410 us in turns; exact, a layer step: 650 -> 644; 14 heads x 32768 of 64, exact, the other way: 2843
           // against 2822)
-          bool pok = nt == 0 || load_k(0);
-          for (int t = 0; t < nt && pok; ++t) pok = (t + 1 >= nt || load_k(t + 1)) && load_v(t);
+          bool pok = tb >= t_end || load_k(tb);
+          for (int t = tb; t < t_end && pok; ++t) pok = (t + 1 >= t_end || load_k(t + 1)) && load_v(t);
           if (!pok) fail_site = 10;
         } else {
-          for (int t = 0; t < nt; ++t)
+          for (int t = tb; t < t_end; ++t)
             if (!load_k(t) || !load_v(t)) { fail_site = 10; break; }
         }
       }
@@ -319,12 +357,12 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
     grid_dependency_wait();
     for (int pass = 0; pass < 2; ++pass) {
-      const int g0 = pass * nt;
+      const int tb = CUT && !pass ? s_part[0] : 0, g0 = (pass ? t_end - (CUT ? s_part[0] : 0) : 0) - tb;
       if (lane == 0) {
         const uint64_t dQ = make_smem_desc_sw128(sQ, 16, 1024);
         bool iok = wait_or_abort(bar(B_QFULL), pass & 1, abortp);
         if (!iok) fail_site = 20;
-        for (int t = 0; t < nt && iok; ++t) {
+        for (int t = tb; t < t_end && iok; ++t) {
           const int g = g0 + t, sb = g & 1, ks = g % KS;
           const int natoms = PipeWord(ld_sched(P.sched + 8 * t)).natoms;
           iok = wait_or_abort(bar(B_KFULL + ks), (g / KS) & 1, abortp);
@@ -355,11 +393,18 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     // =============================== issuer of O += P V ===============================
     asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
     for (int pass = 0; pass < 2; ++pass) {
-      const int g0 = pass * nt;
+      const int tb = CUT && !pass ? s_part[0] : 0, g0 = (pass ? t_end - (CUT ? s_part[0] : 0) : 0) - tb;
       const bool sums = TURNS && pass == 0;  // the whole warp walks the steps, else lane 0 alone
       float sum[2][4] = {};                  // rows 4 lane .. 4 lane + 3, keys 0..63 and 64..127 of the tiles so far
       bool iok = true;
-      for (int t = 0; t < nt && iok && (sums || lane == 0); ++t) {
+      if (CUT && sums && tb > 0 && tb < t_end) {
+        const float* state = cut_state();
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) sum[h][i] = __ldcg(state + T * (D + h) + 4 * lane + i);
+      }
+      for (int t = tb; t < t_end && iok && (sums || lane == 0); ++t) {
         const int g = g0 + t, sb = g & 1, vs = g % VS;
         if (lane == 0) {
           const uint64_t dV = make_smem_desc_sw128(sV + vs * SM::TILE, BLK_BYTES, 1024);
@@ -449,7 +494,7 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       for (int i = 0; i < QW; ++i) w[i] = __byte_perm(x[(QW - 1 - i) >> 1], y[(QW - 1 - i) >> 1], (i & 1) ? 0x5410 : 0x7632);
     };
     for (int pass = 0; pass < 2; ++pass) {
-      const int g0 = pass * nt;
+      const int tb = CUT && !pass ? s_part[0] : 0, g0 = (pass ? t_end - (CUT ? s_part[0] : 0) : 0) - tb;
       const bool safe = pass == 1;
       redone = safe;
       uint32_t qw[QW];
@@ -476,12 +521,12 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         }
       };
       const uint32_t* sched = P.sched + 2 * wq + h;
-      uint32_t e_cur = ld_sched(sched);  // schedule word of the step at hand; the next one is fetched a step ahead
+      uint32_t e_cur = ld_sched(sched + (CUT ? 8 * min(tb, t_end - 1) : 0));  // schedule word of the step at hand; the next one is fetched a step ahead
       int p_mid = PipeWord(e_cur).p_mid;
       if constexpr (SPLIT) {
         if (MODE == ATF_MODE_EXACT) {
           if (ok && !wait_or_abort(bar(B_QFULL), pass & 1, abortp)) { ok = false; fail_site = 30; }
-          if (ok) zero_q_down_to(p_mid);
+          if (ok && (!CUT || tb < t_end)) zero_q_down_to(p_mid);
         }
       } else {
         // ---- Q: this group's half of the pairs of the row, p = h H/2 + i.  Exact mode: what the first MMA does not take
@@ -501,17 +546,40 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         __syncwarp();
         if (lane == 0) {
           mbar_arrive(bar(B_QFULL));
-          if (MODE == ATF_MODE_EXACT && h == 0) mbar_arrive(bar(B_QZ));
+          if (MODE == ATF_MODE_EXACT && h == 0 && (!CUT || tb < t_end)) mbar_arrive(bar(B_QZ));
         }
       }
-      int t = 0;
-      while (t < nt && ok) {
+      if (CUT && tb > 0 && tb < t_end) {  // the second block of a cut tile goes on from what the first left
+        const float* state = cut_state();
+        l_run = __ldcg(state + T * (D + h) + row);
+        m_used = __ldcg(state + T * (D + 2) + row);
+        if (h == 0) {  // O: the first product waits for this group's P
+          const float4* src = reinterpret_cast<const float4*>(state) + row;
+#pragma unroll 1
+          for (int c0 = 0; c0 < D; c0 += 32) {
+            uint32_t o[32];
+#pragma unroll
+            for (int e = 0; e < 32; e += 4) {
+              const float4 v = __ldcg(src + (c0 + e) / 4 * T);
+              o[e] = __float_as_uint(v.x);
+              o[e + 1] = __float_as_uint(v.y);
+              o[e + 2] = __float_as_uint(v.z);
+              o[e + 3] = __float_as_uint(v.w);
+            }
+            tc_st32(tO + c0, o);
+          }
+          tc_wait_st();
+          tc_fence_before();
+        }
+      }
+      int t = tb;
+      while (t < t_end && ok) {
         if constexpr (TURNS) {
           // ---- In turns: behind the diagonal tile group h takes the steps g with g % 2 == h, all 128 keys of its rows. ----
           if (t > 0 && !safe) {
             const float neg_m = -m_used * kScaleLog2;
             const uint32_t tS = tmem_base + h * T + lane_off, tP = tmem_base + 3 * T + h * 64 + lane_off;
-            for (t += (g0 + t + h) & 1; t < nt; t += 2) {
+            for (t += (g0 + t + h) & 1; t < t_end; t += 2) {
               const int g = g0 + t;
               if (!wait_or_abort(bar(B_SFULL + h), (g >> 1) & 1, abortp)) { ok = false; fail_site = 31; break; }
               tc_fence_after();
@@ -550,16 +618,16 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         }
         // ---- plain steps: no mask, no per-cell finish, reference from the diagonal tile.  A loop of its own,
         //      kept small so that it stays in the instruction cache; everything else takes the general step. ----
-        for (; !TURNS && t < nt && !safe && t > 0; ++t) {
+        for (; !TURNS && t < t_end && !safe && t > 0; ++t) {
           const int g = g0 + t, sb = g & 1, ks = g % KS;
           const PipeWord E(e_cur);
           if (!E.plain) break;
-          const uint32_t e_next = t + 1 < nt ? ld_sched(sched + 8 * (t + 1)) : 0u;
+          const uint32_t e_next = t + 1 < t_end ? ld_sched(sched + 8 * (t + 1)) : 0u;
           const int p_all = E.p_all, natoms = E.natoms;
           const int p_mid_next = PipeWord(e_next).p_mid;
           if (!wait_or_abort(bar(B_SFULL + sb), (g >> 1) & 1, abortp)) { ok = false; fail_site = 31; break; }
           tc_fence_after();
-          if (MODE == ATF_MODE_EXACT && t + 1 < nt) zero_q_down_to(p_mid_next);
+          if (MODE == ATF_MODE_EXACT && t + 1 < t_end) zero_q_down_to(p_mid_next);
           float s[64];
           tc_ld32(tmem_base + sb * T + 64 * h + lane_off, reinterpret_cast<uint32_t*>(s));
           tc_ld32(tmem_base + sb * T + 64 * h + lane_off + 32, reinterpret_cast<uint32_t*>(s) + 32);
@@ -585,14 +653,14 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
           p_mid = p_mid_next;
           e_cur = e_next;
         }
-        if (t >= nt || !ok) break;
+        if (t >= t_end || !ok) break;
         // ---- one general step ----
         const int g = g0 + t, sb = g & 1, ks = g % KS;
         const int dt = t;
         const int zrow = dt * T + row;             // distance from this row to column 0 of the key tile
         const int zmax_w = dt * T + 32 * wq + 31 - 64 * h;  // over the warp's 32 x 64 cells
         const PipeWord E(e_cur);
-        const uint32_t e_next = t + 1 < nt ? ld_sched(sched + 8 * (t + 1)) : 0u;
+        const uint32_t e_next = t + 1 < t_end ? ld_sched(sched + 8 * (t + 1)) : 0u;
         const int p_all = E.p_all, p_any = E.p_any, natoms = E.natoms;
         const int p_mid_next = PipeWord(e_next).p_mid;
         const uint32_t tS = tmem_base + sb * T + 64 * h + lane_off;
@@ -600,7 +668,7 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         if (!wait_or_abort(bar(B_SFULL + sb), (g >> 1) & 1, abortp)) { ok = false; fail_site = 31; break; }
         tc_fence_after();
         // S(t) is complete, so Q is not being read: zero what the quarter does not keep in the next tile's MMA
-        if (MODE == ATF_MODE_EXACT && t + 1 < nt) zero_q_down_to(p_mid_next);
+        if (MODE == ATF_MODE_EXACT && t + 1 < t_end) zero_q_down_to(p_mid_next);
         bool s_valid = natoms > 0;  // else no pair is kept in the MMA of this tile and S was not written
         if (MODE == ATF_MODE_EXACT) {
           // ---- per-cell finish.  Pairs [p_all, p_mid) went through the MMA and are not live in every cell of
@@ -809,7 +877,25 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       if (ok && !softmax_sync()) { ok = false; fail_site = 37; }
     }
     const float l_tot = xch[h * 128 + row] + xch[(h ^ 1) * 128 + row];
-    if (ok && nt > 0) {
+    if (CUT && s_part[CUT ? 1 : 0]) {
+      if (ok) {
+        tc_fence_after();
+        float* state = cut_state();
+        float4* dst = reinterpret_cast<float4*>(state) + row;
+#pragma unroll 1
+        for (int q4 = 0; q4 < D / 64; ++q4) {
+          const int c0 = (D / 2) * h + q4 * 32;
+          float o[32];
+          tc_ld32(tO + c0, reinterpret_cast<uint32_t*>(o));
+          tc_wait_ld();
+#pragma unroll
+          for (int e = 0; e < 32; e += 4) __stcg(dst + (c0 + e) / 4 * T, make_float4(o[e], o[e + 1], o[e + 2], o[e + 3]));
+        }
+        state[T * (D + h) + row] = xch[h * 128 + row];
+        if (h == 0) state[T * (D + 2) + row] = m_used;
+      }
+      __threadfence();
+    } else if (ok) {
       tc_fence_after();
       const float inv = 1.f / l_tot;
       __nv_bfloat16* orow = P.O + qrow * D;
@@ -846,27 +932,46 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   }
   tc_fence_before();
   __syncthreads();
+  if (CUT && tid == 0 && s_part[CUT ? 1 : 0] && !s_abort) st_release(P.flags + blockIdx.x, s_redo ? 2u : 1u);
   if (warp == 0) tmem_dealloc(tmem_base, TMEM_COLS);
 }
 
 template <int D, bool SPLIT>
 atf_status launch_pipe(const CUtensorMap& tq, const CUtensorMap& tql, const CUtensorMap& tk, const CUtensorMap& tkl,
-                       const CUtensorMap& tv, const AtfPipeParams& P, const AtfTable& t, int B, int mode, bool count,
+                       const CUtensorMap& tv, AtfPipeParams P, const AtfTable& t, int B, int mode, bool count,
                        cudaStream_t s) {
-  const int ntq = (P.N + T - 1) / T;
-  const int it0 = (P.N - P.Nq) / T;  // first tile with a query row
+  const int tiles = (P.N + T - 1) / T - (P.N - P.Nq) / T;  // from the first one with a query row
   cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(ntq - it0, P.Hq, B);
+  // Order of the tiles.  Rows of different lengths: longest first over all heads, so that no head's longest row starts when the
+  // others are done (us, head by head -> so: a layer step of 24 heads x 8192 rows 642 -> 634, 3000 rows 172 -> 141, 14 heads x
+  // 1200 of 64 26.4 -> 21.3), in equal groups of heads whose K and V stay in L2 together.  Rows of about the same length: head
+  // by head (B = 2, 24 heads, 2048 rows of 8192: 457, over all heads 470; 2 x 2 heads, 16000 of 60000: 1226 against 1265).
+  const int64_t dlim = ((int64_t)t.w[D / 2 - 1] + T - 1) / T + 1, per_kv = P.Hq / P.Hkv;
+  const int64_t longest = std::min<int64_t>((P.N + T - 1) / T, dlim), shortest = std::min<int64_t>((P.N - P.Nq) / T + 1, dlim);
+  P.heads = P.Hq * B;
+  int64_t group = 1;
+  if (P.cuts) {
+    group = P.heads;
+  } else if (2 * shortest <= longest) {
+    const int64_t fit = std::max<int64_t>(1, (64ll << 20) / ((int64_t)P.N * D * 2 * (SPLIT ? 3 : 2))) * per_kv;
+    const int64_t groups = (P.heads + fit - 1) / fit;
+    group = std::min<int64_t>(((P.heads + groups - 1) / groups + per_kv - 1) / per_kv * per_kv, P.heads);
+  }
+  P.group = (int)std::max<int64_t>(group, (P.heads + 65534) / 65535);  // gridDim.y
+  P.jobs = tiles * P.group;
+  if ((int64_t)tiles * P.group > 0x7FFFFF00) return atf_fail(ATF_ERR_UNSUPPORTED, "atf_prefill: problem too large for the grid");
+  cfg.gridDim = dim3((unsigned)(P.jobs + P.cuts), (P.heads + P.group - 1) / P.group);
   cfg.stream = s;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
   cfg.blockDim = dim3(PP_THREADS);
 #define ATF_PP_LAUNCH(MODE_, COUNT_, TURNS_)                                                          \
   do {                                                                                                 \
-    auto kern = atf_prefill_pipe_kernel<D, MODE_, COUNT_, SPLIT, TURNS_>;                              \
+    auto kern = P.cuts && !COUNT_ ? atf_prefill_pipe_kernel<D, MODE_, COUNT_, SPLIT, TURNS_, !COUNT_>  \
+                                  : atf_prefill_pipe_kernel<D, MODE_, COUNT_, SPLIT, TURNS_, false>;   \
     const int smem = PipeSmem<D, SPLIT, MODE_ == ATF_MODE_EXACT && !SPLIT, TURNS_>::DYN_BYTES;                 \
     ATF_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));     \
     cfg.dynamicSmemBytes = smem;                                                                       \

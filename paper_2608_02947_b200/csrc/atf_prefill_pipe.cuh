@@ -2,6 +2,8 @@
 // atf_prefill.cu and atf_prefill_split.cu (validation, pre-pass, tensor maps) calls it.
 #pragma once
 
+#include <algorithm>
+
 #include "atf_common.cuh"
 
 struct AtfPipeParams {
@@ -16,6 +18,11 @@ struct AtfPipeParams {
   int Hq, Hkv;
   int N;   // number of keys; positions 0..N-1
   int Nq;  // number of query rows: the last Nq positions
+  int heads, group;     // all heads (B Hq), heads whose tiles are dealt out together
+  int jobs;             // tiles of a group
+  int cuts;             // tiles that two blocks share, atf_prefill_cuts()
+  unsigned int* flags;  // [cuts], zeroed by the pre-pass
+  float* state;         // [cuts][128 (d + 3)]
 };
 
 atf_status atf_launch_prefill_pipe(const CUtensorMap& tk, const CUtensorMap& tv, const AtfPipeParams& P,
@@ -28,6 +35,27 @@ atf_status atf_launch_prefill_pipe_split(const CUtensorMap& tqh, const CUtensorM
 // The pre-pass of a prefill (layout of K and the band schedule) is one launch of blocks of this many threads: the first
 // atf_sched_blocks() write the schedule, the others move rows.
 constexpr int ATF_PREP_THREADS = 256;
+// Cut tiles.  Rows of about the same length in few waves leave the SMs idle at the end (32 tiles of 445 to 477 steps for each of
+// 24 heads are 5.2 waves that run as 6).  Then the first ATF_SMS tiles are worked on by two blocks each: blocks 0 .. ATF_SMS - 1
+// take the first (j + 1/2) / ATF_SMS of tile j's steps, which lets the SMs fall out of step evenly, and the blocks behind all
+// others go on where those stopped, the longest rest first, so that all SMs end together.  O, row sums and reference pass
+// through memory in fp32 as they stand: the result is bit for bit that of one block.  A block waits for one that started
+// before it, at a time when that one is long done.
+// Cut where the idle share is above a fifth: the kernel with the cut is 2 to 4 % slower, rows out of step share fewer K and V
+// tiles in L2, and under the power cap idle SMs leave their power to the others (us, whole -> cut: 2000 of 20000, 14 heads of 64,
+// 24 % idle, exact 274 -> 250, coarse 226 -> 211; 24 heads of 128, 1000 of 12000, 37 %, 222 -> 208, 1000 of 100000, full, 37 %,
+// 1601 -> 1343; but 4000 of 61003, coarse, 15 %, 2510 -> 2516).
+constexpr int ATF_SMS = 148;
+inline size_t atf_cut_floats(int d) { return (size_t)ATF_SMS * 128 * (d + 3); }
+inline int atf_prefill_cuts(int64_t N, int64_t Nq, int64_t heads, int w_max, int d, size_t spare_bytes) {
+  const int64_t dlim = ((int64_t)w_max + 127) / 128 + 1, last = (N + 127) / 128, first = (N - Nq) / 128;
+  const int64_t jobs = (last - first) * heads, waves = (jobs + ATF_SMS - 1) / ATF_SMS;
+  if (jobs <= ATF_SMS || jobs > 0x7FFFFF00 || spare_bytes < (atf_cut_floats(d) + ATF_SMS) * 4) return 0;
+  // steps of a block: its key tiles, and three for prologue and epilogue
+  const int64_t shortest = std::min(first + 1, dlim) + 3, longest = std::min(last, dlim) + 3;
+  const double busy = (double)jobs * (shortest + longest) / 2, idle = (double)(waves * ATF_SMS - jobs) * shortest;
+  return idle > 0.2 * busy + 12 * ATF_SMS ? ATF_SMS : 0;
+}
 inline int atf_sched_blocks(int64_t N) { return (int)(((N + 127) / 128 + ATF_PREP_THREADS / 8 - 1) / (ATF_PREP_THREADS / 8)); }
 
 #ifdef __CUDACC__
@@ -39,9 +67,21 @@ __device__ __forceinline__ uint32_t ld_sched(const uint32_t* p) {
   return w;
 }
 
+// The flag between the two blocks of a cut tile.
+__device__ __forceinline__ unsigned int ld_acquire(const unsigned int* p) {
+  unsigned int v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_release(unsigned int* p, unsigned int v) {
+  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
 // Schedule words of PREP_THREADS / 8 tile distances, one word a thread (8 (row quarter, key half) blocks for each; see
 // PipeWord in atf_prefill_pipe.cu).
-__device__ inline void atf_write_schedule(const AtfTable& table, int mode, int H, int ndt, uint32_t* __restrict__ out) {
+__device__ inline void atf_write_schedule(const AtfTable& table, int mode, int H, int ndt, uint32_t* __restrict__ out, int cuts,
+                                          unsigned int* __restrict__ flags) {
+  if (blockIdx.x == 0 && (int)threadIdx.x < cuts) flags[threadIdx.x] = 0u;
   constexpr int T = 128;
   __shared__ int w[ATF_MAX_PAIRS];
   if (threadIdx.x < H) w[threadIdx.x] = table.w[threadIdx.x];

@@ -27,13 +27,14 @@ constexpr int T = 128;
 // column order.  One thread moves eight pairs of a row; memory bounds it (10001 rows of 24 + 8 heads of 128: 49 us, 327 MB).
 __global__ void __launch_bounds__(ATF_PREP_THREADS)
 atf_split_prep_kernel(const __grid_constant__ AtfTable table, int mode, int ndt, int sched_blocks, uint32_t* __restrict__ sched,
+                      int cuts, unsigned int* __restrict__ flags,
                       const float* __restrict__ Q, const float* __restrict__ K, __nv_bfloat16* __restrict__ Qhi,
                       __nv_bfloat16* __restrict__ Qlo, __nv_bfloat16* __restrict__ Khi, __nv_bfloat16* __restrict__ Klo,
                       int64_t rows_q, int64_t rows_k, int D) {
   grid_dependency_wait();
   grid_dependency_launch();
   const int H = D / 2, per_row = D / 16;
-  if ((int)blockIdx.x < sched_blocks) return atf_write_schedule(table, mode, H, ndt, sched);
+  if ((int)blockIdx.x < sched_blocks) return atf_write_schedule(table, mode, H, ndt, sched, cuts, flags);
   const int64_t gid = (int64_t)(blockIdx.x - sched_blocks) * ATF_PREP_THREADS + threadIdx.x;
   int64_t row = gid / per_row;
   const int c = (int)(gid % per_row);           // dims 8c .. 8c + 7 of each half, pairs 8j .. 8j + 7 in falling order
@@ -114,6 +115,10 @@ extern "C" atf_status atf_prefill_split_chunk(const float* Q, const float* K, co
   __nv_bfloat16* Khi = (__nv_bfloat16*)(parts + 2 * qb);
   __nv_bfloat16* Klo = (__nv_bfloat16*)(parts + 2 * qb + kb);
   cudaStream_t s = (cudaStream_t)stream;
+  const size_t used = ATF_WS_HEADER + split_sched_bytes(N) + 2 * (qb + kb);  // `need` is that of N query rows
+  const int cuts = opts && opts->kept_terms ? 0 : atf_prefill_cuts(N, Nq, (int64_t)B * Hq, t.w[d / 2 - 1], d, ws.bytes - used);
+  float* state = (float*)(base + used);
+  unsigned int* flags = (unsigned int*)(state + atf_cut_floats(d));
   {
     const int64_t rows_q = (int64_t)B * Hq * Nq, rows_k = (int64_t)B * Hkv * N;
     if ((rows_q * (d / 8) + 255) / 256 > 0x7FFFFFFF) return atf_fail(ATF_ERR_UNSUPPORTED, "atf_prefill_split: problem too large for the repack grid");
@@ -121,7 +126,7 @@ extern "C" atf_status atf_prefill_split_chunk(const float* Q, const float* K, co
     const int64_t blocks = sb + ((rows_q + rows_k) * (d / 16) + ATF_PREP_THREADS - 1) / ATF_PREP_THREADS;
     if (blocks > 0x7FFFFFFF) return atf_fail(ATF_ERR_UNSUPPORTED, "atf_prefill_split: problem too large for the repack grid");
     ATF_CUDA_CHECK(atf_launch_overlapped(atf_split_prep_kernel, dim3((unsigned)blocks), ATF_PREP_THREADS, 0, s, t, mode, (int)((N + T - 1) / T), sb,
-                                                                        (uint32_t*)(base + ATF_WS_HEADER), Q, K, Qhi, Qlo, Khi,
+                                                                        (uint32_t*)(base + ATF_WS_HEADER), cuts, flags, Q, K, Qhi, Qlo, Khi,
                                                                         Klo, rows_q, rows_k, d));
   }
   CUtensorMap tqh, tql, tkh, tkl, tv;
@@ -138,6 +143,9 @@ extern "C" atf_status atf_prefill_split_chunk(const float* Q, const float* K, co
   P.Qlo = Qlo;
   P.O = (__nv_bfloat16*)O;
   P.LSE = LSE;
+  P.cuts = cuts;
+  P.flags = flags;
+  P.state = state;
   P.kept = opts ? (unsigned long long*)opts->kept_terms : nullptr;
   P.status = (unsigned int*)base;
   P.Hq = Hq;

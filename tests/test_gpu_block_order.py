@@ -1,0 +1,53 @@
+"""How a prefill's tiles are dealt to blocks: groups of heads (a whole one, a ragged last one), and tiles that two blocks share."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+# rows of different lengths; keys and values of a KV head: 36 MB (one a group), 13 MB (two groups, the last one short); split
+# mode: 27 MB (two groups, the last one short); rows of about the same length: head by head
+@pytest.mark.parametrize("B,Hq,Hkv,N,Nq,d,split", [(3, 6, 2, 70000, 36000, 128, False), (7, 2, 1, 50000, 26000, 64, False),
+                                                   (3, 3, 1, 35000, 18000, 128, True), (2, 6, 2, 9000, 300, 128, False)])
+def test_heads_in_groups(B, Hq, Hkv, N, Nq, d, split):
+    import paper_2608_02947_b200 as atf
+    g = torch.Generator(device="cuda").manual_seed(N)
+    kind = torch.float32 if split else torch.bfloat16
+    Q, K, V = [torch.randn((B, h, n, d), generator=g, device="cuda").to(t) for h, n, t in ((Hq, Nq, kind), (Hkv, N, kind), (Hkv, N, torch.bfloat16))]
+    W, _ = atf.atf_window_table(5e5, d, 2.0, N)
+    call = atf.atf_prefill_split if split else atf.atf_prefill
+    O, lse = call(Q, K, V, table=W)
+    for b in range(B):
+        for k in range(Hkv):
+            h = slice(k * Hq // Hkv, (k + 1) * Hq // Hkv)
+            o, l = call(Q[b:b + 1, h].contiguous(), K[b:b + 1, k:k + 1].contiguous(), V[b:b + 1, k:k + 1].contiguous(), table=W)
+            assert torch.equal(O[b:b + 1, h], o) and torch.equal(lse[b:b + 1, h], l)
+    atf.binding.check_status()
+
+
+# Bit for bit what one block gives (a call that counts terms never cuts): just above one wave of blocks, an odd number of waves,
+# ragged rows, windows that end (equal short tiles), the safe second pass seen in front of the cut and behind it, the split form
+@pytest.mark.parametrize("B,Hq,Hkv,N,Nq,d,mode,far,split", [
+    (1, 24, 8, 9000, 850, 128, 0, 0, False), (2, 14, 2, 12345, 700, 64, 0, 0, False), (1, 24, 8, 30000, 1111, 128, 1, 0, False),
+    (1, 40, 8, 9000, 512, 128, 0, 1, False), (1, 40, 8, 9000, 512, 64, 0, 2, False), (1, 40, 8, 9000, 512, 128, 1, 2, False),
+    (3, 14, 2, 20000, 500, 64, 1, 3, False), (1, 24, 8, 9000, 850, 128, 0, 0, True), (1, 40, 8, 9000, 512, 128, 0, 2, True)])
+def test_cut_tiles(B, Hq, Hkv, N, Nq, d, mode, far, split):
+    import paper_2608_02947_b200 as atf
+    g = torch.Generator(device="cuda").manual_seed(N + far)
+    kind = torch.float32 if split else torch.bfloat16
+    Q, K, V = [torch.randn((B, h, n, d), generator=g, device="cuda") for h, n in ((Hq, Nq), (Hkv, N), (Hkv, N))]
+    W, _ = atf.atf_window_table(5e5, d, 2.0, N)
+    if far == 3:  # no pair reaches further: every tile has the same few steps
+        W = W.clamp(max=7000)
+    elif far:     # logits that the reference of the diagonal tile cannot hold, in near (1) or far (2) keys
+        K[:, :, slice(N - 2000, N - 1500) if far == 1 else slice(0, 500)] *= 30
+        Q *= 4
+    Q, K, V = Q.to(kind), K.to(kind), V.to(torch.bfloat16)
+    call = atf.atf_prefill_split if split else atf.atf_prefill
+    # room for the state of the cut tiles beside what the call asks for
+    atf.ensure_workspace(3 * atf.atf_workspace_bytes(atf.binding.ATF_OP_PREFILL, B, Hq, Hkv, N, d), "cuda:0")
+    whole = call(Q, K, V, table=W, mode=mode, kept_terms=torch.zeros(B * Hq, dtype=torch.int64, device="cuda"))
+    for _ in range(3):
+        O, lse = call(Q, K, V, table=W, mode=mode)
+        assert torch.equal(O, whole[0]) and torch.equal(lse, whole[1])
+    atf.binding.check_status()
