@@ -26,11 +26,13 @@ constexpr int T = 128;  // query rows per tile and key columns per tile
 // first n_per_head are copied, the result is dense.
 // With Kg the same eight pairs, a group of the tiled group-major K cache (kg_tiles tiles per head), also go there for the
 // rows from kg_first_row on.
+// X may be what a rotation that still runs is writing (launch: atf_launch_overlapped), so no pointer is __restrict__: the loads
+// are ordinary ones and stay behind the wait.
 __global__ void __launch_bounds__(ATF_PREP_THREADS)
-atf_prefill_prep_kernel(const __grid_constant__ AtfTable table, int mode, int ndt, int sched_blocks, uint32_t* __restrict__ sched,
-                        int cuts, unsigned int* __restrict__ flags,
-                        const __nv_bfloat16* __restrict__ X, __nv_bfloat16* __restrict__ Y, int64_t rows, int D,
-                        int64_t n_per_head, int64_t src_head_rows, __nv_bfloat16* __restrict__ Kg, int64_t kg_tiles,
+atf_prefill_prep_kernel(const __grid_constant__ AtfTable table, int mode, int ndt, int sched_blocks, uint32_t* sched,
+                        int cuts, unsigned int* flags,
+                        const __nv_bfloat16* X, __nv_bfloat16* Y, int64_t rows, int D,
+                        int64_t n_per_head, int64_t src_head_rows, __nv_bfloat16* Kg, int64_t kg_tiles,
                         int64_t kg_first_row) {
   grid_dependency_wait();  // before the prefill kernel may start: it reads Q ahead of its own wait
   grid_dependency_launch();

@@ -79,8 +79,8 @@ __device__ __forceinline__ void st_release(unsigned int* p, unsigned int v) {
 
 // Schedule words of PREP_THREADS / 8 tile distances, one word a thread (8 (row quarter, key half) blocks for each; see
 // PipeWord in atf_prefill_pipe.cu).
-__device__ inline void atf_write_schedule(const AtfTable& table, int mode, int H, int ndt, uint32_t* __restrict__ out, int cuts,
-                                          unsigned int* __restrict__ flags) {
+__device__ inline void atf_write_schedule(const AtfTable& table, int mode, int H, int ndt, uint32_t* out, int cuts,
+                                          unsigned int* flags) {
   if (blockIdx.x == 0 && (int)threadIdx.x < cuts) flags[threadIdx.x] = 0u;
   constexpr int T = 128;
   __shared__ int w[ATF_MAX_PAIRS];

@@ -83,3 +83,52 @@ def test_captured_chain():
         torch.cuda.synchronize()
         for a, b in zip(want, got):
             assert torch.equal(a, b)
+
+
+def _queued(steps, rounds):
+    """steps(i) for every round: with a synchronisation behind each call, queued behind a kernel that keeps the GPU busy (the
+    host is ahead, so the kernels follow one another as closely as they can), and captured in a graph."""
+    want = [steps(i, torch.cuda.synchronize) for i in range(rounds)]
+    torch.cuda.synchronize()
+    for _ in range(5):
+        torch.cuda._sleep(20_000_000)
+        got = [steps(i, lambda: None) for i in range(rounds)]
+        torch.cuda.synchronize()
+        for a, b in zip(want, got):
+            assert all(torch.equal(x, y) for x, y in zip(a, b))
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        got = [steps(i, lambda: None) for i in range(rounds)]
+    for _ in range(3):
+        graph.replay()
+        torch.cuda.synchronize()
+        for a, b in zip(want, got):
+            assert all(torch.equal(x, y) for x, y in zip(a, b))
+
+
+# Q and K rotated right before the call that reads them, other values in the same buffers each time: a read in front of the wait,
+# or one that the read-only path kept from the round before, would give other bits
+@pytest.mark.parametrize("d,Hkv,N,Nq,mode", [(128, 8, 3000, 3000, 0), (128, 8, 3000, 400, 1), (64, 2, 12000, 12000, 1), (64, 3, 700, 700, 0)])
+def test_rotation_then_prefill(d, Hkv, N, Nq, mode):
+    import paper_2608_02947_b200 as atf
+    g = torch.Generator(device="cuda").manual_seed(N + Nq)
+    W, theta = atf.atf_window_table(5e5, d, 2.0, N)
+    table = atf.WindowTable(W)
+    Qs, Ks, Vs = [[torch.randn((1, h, n, d), generator=g, device="cuda").to(torch.bfloat16) for _ in range(3)]
+                  for h, n in ((2 * Hkv, Nq), (Hkv, N), (Hkv, N))]
+    Q, K, V = Qs[0].clone(), Ks[0].clone(), Vs[0].clone()
+    cache = atf.new_kcache_groups(1, Hkv, N, d, "cuda")
+
+    def steps(i, wait):
+        for x, src in ((Q, Qs), (K, Ks), (V, Vs)):
+            x.copy_(src[i])
+        wait()
+        atf.atf_rope(Q, theta, pos0=N - Nq)
+        wait()
+        atf.atf_rope(K, theta)
+        wait()
+        O, lse = atf.atf_prefill(Q, K, V, table=table, mode=mode, kcache_groups=cache)
+        wait()
+        return O, lse, cache.clone()
+
+    _queued(steps, 3)

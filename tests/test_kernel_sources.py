@@ -1,0 +1,51 @@
+"""Rules of the kernels that a run need not show to be broken, checked in the sources."""
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2608_02947_b200", "csrc")
+
+
+def _code():
+    text = "".join(open(os.path.join(CSRC, f)).read() for f in sorted(os.listdir(CSRC)))
+    return re.sub(r"//[^\n]*|/\*.*?\*/", "", text, flags=re.S)
+
+
+def _closed(text, i, pair):
+    """End of the bracket that opens at text[i]."""
+    depth = 0
+    while True:
+        depth += (text[i] == pair[0]) - (text[i] == pair[1])
+        i += 1
+        if depth == 0:
+            return i
+
+
+def _function(code, name):
+    """Parameters and body of the function of this name."""
+    for m in re.finditer(r"\b" + name + r"\s*\(", code):
+        end = _closed(code, m.end() - 1, "()")
+        if code[end:].lstrip().startswith("{"):
+            body = code.index("{", end)
+            return code[m.end():end - 1], code[body:_closed(code, body, "{}")]
+    raise AssertionError(f"{name} has no definition")
+
+
+# A kernel that starts while its predecessor still writes waits before it reads.  That order holds for ordinary loads only: __ldg,
+# and a load through a __restrict__ parameter, which the compiler may take for the read-only path, are for memory that nothing
+# writes while the kernel is resident, and may be moved over the wait.
+OVERLAPPED = ["atf_prefill_prep_kernel"]
+
+
+@pytest.mark.parametrize("kernel", OVERLAPPED)
+def test_reads_behind_the_wait_stay_there(kernel):
+    code = _code()
+    parameters, body = _function(code, kernel)
+    assert "grid_dependency_wait()" in body
+    for helper in ("atf_write_schedule", "merge_splits"):
+        if helper in body:
+            p, b = _function(code, helper)
+            parameters, body = parameters + p, body + b
+    assert "__restrict__" not in parameters
+    assert "__ldg" not in body and "ld.global.nc" not in body
