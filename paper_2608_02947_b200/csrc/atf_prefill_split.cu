@@ -25,11 +25,12 @@ constexpr int T = 128;
 
 // The pre-pass, one launch: band schedule, then hi = bf16(x), lo = bf16(x - hi) of Q and of K in the pair-interleaved
 // column order.  One thread moves eight pairs of a row; memory bounds it (10001 rows of 24 + 8 heads of 128: 49 us, 327 MB).
+// Q and K may be what a rotation that still runs is writing: no pointer is __restrict__, the loads stay behind the wait.
 __global__ void __launch_bounds__(ATF_PREP_THREADS)
-atf_split_prep_kernel(const __grid_constant__ AtfTable table, int mode, int ndt, int sched_blocks, uint32_t* __restrict__ sched,
-                      int cuts, unsigned int* __restrict__ flags,
-                      const float* __restrict__ Q, const float* __restrict__ K, __nv_bfloat16* __restrict__ Qhi,
-                      __nv_bfloat16* __restrict__ Qlo, __nv_bfloat16* __restrict__ Khi, __nv_bfloat16* __restrict__ Klo,
+atf_split_prep_kernel(const __grid_constant__ AtfTable table, int mode, int ndt, int sched_blocks, uint32_t* sched,
+                      int cuts, unsigned int* flags,
+                      const float* Q, const float* K, __nv_bfloat16* Qhi,
+                      __nv_bfloat16* Qlo, __nv_bfloat16* Khi, __nv_bfloat16* Klo,
                       int64_t rows_q, int64_t rows_k, int D) {
   grid_dependency_wait();
   grid_dependency_launch();

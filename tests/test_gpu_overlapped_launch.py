@@ -132,3 +132,27 @@ def test_rotation_then_prefill(d, Hkv, N, Nq, mode):
         return O, lse, cache.clone()
 
     _queued(steps, 3)
+
+
+@pytest.mark.parametrize("d,Hkv,N,Nq,mode", [(128, 4, 3000, 3000, 0), (64, 2, 9000, 500, 1)])
+def test_rotation_then_split_prefill(d, Hkv, N, Nq, mode):
+    import paper_2608_02947_b200 as atf
+    g = torch.Generator(device="cuda").manual_seed(N + Nq)
+    W, theta = atf.atf_window_table(5e5, d, 2.0, N)
+    table = atf.WindowTable(W)
+    Qs, Ks = [[torch.randn((1, h, n, d), generator=g, device="cuda") for _ in range(3)] for h, n in ((2 * Hkv, Nq), (Hkv, N))]
+    Vs = [torch.randn((1, Hkv, N, d), generator=g, device="cuda").to(torch.bfloat16) for _ in range(3)]
+    Q, K, V = Qs[0].clone(), Ks[0].clone(), Vs[0].clone()
+
+    def steps(i, wait):
+        for x, src in ((Q, Qs), (K, Ks), (V, Vs)):
+            x.copy_(src[i])
+        for x, pos in ((K, 0), (Q, N - Nq)) if i == 1 else ((Q, N - Nq), (K, 0)):
+            wait()
+            atf.atf_rope_f32(x, theta, pos0=pos)
+        wait()
+        out = atf.atf_prefill_split(Q, K, V, table=table, mode=mode)
+        wait()
+        return out
+
+    _queued(steps, 3)
