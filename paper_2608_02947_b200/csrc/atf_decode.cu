@@ -677,7 +677,7 @@ atf_decode_tiles_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_co
 #pragma unroll
           for (int kp = 0; kp < NKG / 2; ++kp) {
             const float2* src = P.rot_key + (8 * j + 4 * c + t4) * KT + warp * KB + 16 * kp + g;
-            const float2 k0 = __ldg(src), k1 = __ldg(src + 8);
+            const float2 k0 = src[0], k1 = src[8];  // ordinary loads: the tables' kernel may be the one before this
             kc[j][c][kp] = make_float2(k0.x, k1.x);
             ksi[j][c][kp] = make_float2(k0.y, k1.y);
           }

@@ -156,3 +156,36 @@ def test_rotation_then_split_prefill(d, Hkv, N, Nq, mode):
         return out
 
     _queued(steps, 3)
+
+
+@pytest.mark.parametrize("d,G,L", [(128, 3, 5000), (64, 7, 300)])
+def test_tables_then_decode(d, G, L):
+    """Rotation tables of another base in the same buffer, built right before the decode that reads them."""
+    import ctypes as C
+
+    import paper_2608_02947_b200 as atf
+    g = torch.Generator(device="cuda").manual_seed(L)
+    K, V = [torch.randn((2, 2, L, d), generator=g, device="cuda").to(torch.bfloat16) for _ in range(2)]
+    q = torch.randn((2, 2 * G, d), generator=g, device="cuda").to(torch.bfloat16)
+    cache = atf.atf_kcache_pack(K)
+    W, _ = atf.atf_window_table(5e5, d, 2.0, L)
+    table = atf.WindowTable(W)
+    thetas = [atf.atf_window_table(base, d, 2.0, L)[1] for base in (1e4, 5e5, 1e7)]
+    tables = atf.atf_rope_tables(thetas[0], d, L)
+
+    def steps(i, wait):
+        arr = (C.c_double * (d // 2))(*thetas[i].tolist())
+        atf.binding._check(atf.lib().atf_rope_tables(arr, d, 7 * i, L, C.c_void_p(tables.buf.data_ptr()), tables.buf.numel(),
+                                                     C.c_void_p(torch.cuda.current_stream().cuda_stream)))
+        wait()
+        x = q.clone()
+        atf.atf_rope(x[:, :, None], thetas[i], pos0=7 * i + L - 1)
+        wait()
+        out = atf.atf_decode(x, cache, V, table=table, return_lse=True, rope_tables=tables)
+        wait()
+        atf.binding._check(atf.lib().atf_rope_tables(arr, d, 7 * i + 1, L, C.c_void_p(tables.buf.data_ptr()), tables.buf.numel(),
+                                                     C.c_void_p(torch.cuda.current_stream().cuda_stream)))
+        wait()
+        return out + atf.atf_decode(x, cache, V, table=table, return_lse=True, rope_tables=tables)
+
+    _queued(steps, 3)

@@ -35,7 +35,7 @@ def _function(code, name):
 # A kernel that starts while its predecessor still writes waits before it reads.  That order holds for ordinary loads only: __ldg,
 # and a load through a __restrict__ parameter, which the compiler may take for the read-only path, are for memory that nothing
 # writes while the kernel is resident, and may be moved over the wait.
-OVERLAPPED = ["atf_prefill_prep_kernel", "atf_split_prep_kernel"]
+OVERLAPPED = ["atf_prefill_prep_kernel", "atf_split_prep_kernel", "atf_decode_kernel", "atf_decode_tiles_kernel"]
 
 
 @pytest.mark.parametrize("kernel", OVERLAPPED)
