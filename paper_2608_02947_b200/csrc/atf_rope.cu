@@ -49,7 +49,7 @@ __device__ __forceinline__ void store8(float* p, const double (&v)[8]) {
 // PRE: the next head's segment is loaded before this one is stored, for fp32 data that L2 does not hold.
 constexpr int ROPE_THREADS = 256;
 template <int D, int HL, typename T, bool SPREAD = false, bool PRE = false>
-__global__ void __launch_bounds__(ROPE_THREADS) atf_rope_kernel(T* __restrict__ X, int BH, int64_t N, int64_t pos0,
+__global__ void __launch_bounds__(ROPE_THREADS) atf_rope_kernel(T* X, int BH, int64_t N, int64_t pos0,
                                                                 const __grid_constant__ RopeTheta theta) {
   constexpr int H = D / 2;
   constexpr int CHUNKS = H / 8;                         // segments of 8 pairs per row
@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(ROPE_THREADS) atf_rope_kernel(T* __restrict__ 
     store8(row, olo);
     store8(row + H, ohi);
   };
-  grid_dependency_wait();  // the angles need nothing of the kernel before
+  grid_dependency_wait();  // the angles need nothing of the kernel before; X, not __restrict__, is touched behind this alone
   const int64_t head = N * D;
   const int lane = threadIdx.x / SEGS;
   const int first = SPREAD ? (int)blockIdx.y * HL + lane : lane, step = SPREAD ? HL * (int)gridDim.y : HL;

@@ -189,3 +189,25 @@ def test_tables_then_decode(d, G, L):
         return out + atf.atf_decode(x, cache, V, table=table, return_lse=True, rope_tables=tables)
 
     _queued(steps, 3)
+
+
+@pytest.mark.parametrize("f32", [False, True])
+@pytest.mark.parametrize("d,H,N", [(128, 8, 9000), (64, 24, 1), (128, 32, 130)])
+def test_rotations_in_a_row(d, H, N, f32):
+    """In place, each on what the one before it wrote."""
+    import paper_2608_02947_b200 as atf
+    g = torch.Generator(device="cuda").manual_seed(N)
+    _, theta = atf.atf_window_table(5e5, d, 2.0, N)
+    src = torch.randn((3, H, N, d), generator=g, device="cuda")
+    src = src if f32 else src.to(torch.bfloat16)
+    X = src[:1].clone()
+
+    def steps(i, wait):
+        X.copy_(src[i:i + 1])
+        for pos in (0, 3, 1000, 77):
+            wait()
+            (atf.atf_rope_f32 if f32 else atf.atf_rope)(X, theta, pos0=pos + i)
+        wait()
+        return X.clone(),
+
+    _queued(steps, 3)

@@ -35,7 +35,8 @@ def _function(code, name):
 # A kernel that starts while its predecessor still writes waits before it reads.  That order holds for ordinary loads only: __ldg,
 # and a load through a __restrict__ parameter, which the compiler may take for the read-only path, are for memory that nothing
 # writes while the kernel is resident, and may be moved over the wait.
-OVERLAPPED = ["atf_prefill_prep_kernel", "atf_split_prep_kernel", "atf_decode_kernel", "atf_decode_tiles_kernel"]
+OVERLAPPED = ["atf_prefill_prep_kernel", "atf_split_prep_kernel", "atf_decode_kernel", "atf_decode_tiles_kernel", "atf_prefill_pipe_kernel",
+              "atf_rope_kernel"]
 
 
 @pytest.mark.parametrize("kernel", OVERLAPPED)
@@ -49,3 +50,11 @@ def test_reads_behind_the_wait_stay_there(kernel):
             parameters, body = parameters + p, body + b
     assert "__restrict__" not in parameters
     assert "__ldg" not in body and "ld.global.nc" not in body
+
+
+def test_every_overlapped_kernel_is_looked_at():
+    """A kernel is launched either in the ordinary way or by one of the two calls that set the attribute."""
+    code = _code()
+    kernels = set(re.findall(r"\b(atf_\w+_kernel)\b", code))
+    assert set(OVERLAPPED) == {k for k in kernels if not re.search(k + r"\s*<<<", code)}
+    assert len(kernels) > len(OVERLAPPED) and len(re.findall(r"ProgrammaticStreamSerialization;", code)) == 2
