@@ -425,6 +425,7 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
           // the tile's sums, added in the order of the tiles
           iok = __shfl_sync(0xffffffffu, (int)iok, 0);
           if (!iok) break;
+          __syncwarp();  // lane 0 alone has waited for what the softmax warps wrote, and a shuffle orders no memory
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             float v[4];

@@ -58,3 +58,11 @@ def test_every_overlapped_kernel_is_looked_at():
     kernels = set(re.findall(r"\b(atf_\w+_kernel)\b", code))
     assert set(OVERLAPPED) == {k for k in kernels if not re.search(k + r"\s*<<<", code)}
     assert len(kernels) > len(OVERLAPPED) and len(re.findall(r"ProgrammaticStreamSerialization;", code)) == 2
+
+
+def test_sums_are_read_behind_a_barrier_of_the_warp():
+    """In turns one lane waits for a tile's sums and the whole warp reads them: a shuffle passes a value on, not the order of memory."""
+    _, body = _function(_code(), "atf_prefill_pipe_kernel")
+    wait = body.index("bar(B_PFULL + 2 * sb + h)")
+    between = body[body.index("__shfl_sync", wait):body.index("lds_f4(", wait)]
+    assert "__syncwarp();" in between
