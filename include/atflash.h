@@ -325,8 +325,8 @@ atf_status atf_check_status(void* stream);
 atf_status atf_check_status_at(void* workspace, void* stream);
 
 /* Self-test of that report path: launches one small kernel that waits, with the kernels' bounded
- * wait and a limit of limit_us microseconds (1..100000), for a barrier nobody signals, gives up
- * and records it in the bound workspace.  The next atf_check_status returns ATF_ERR_TIMEOUT once. */
+ * waits and a limit of limit_us microseconds (1..100000) each, for a barrier nobody signals and
+ * for a flag nobody sets, gives up and records it in the bound workspace.  The next atf_check_status returns ATF_ERR_TIMEOUT once. */
 atf_status atf_selftest_bounded_wait(unsigned int limit_us, void* stream);
 
 /* Diagnostic behind the choice of K-cache layouts: reads `bytes` of device memory as 256-byte rows (a K row

@@ -101,8 +101,8 @@ atf_status atf_validate_table(const char* who, const int64_t* table, int d, int6
   return ATF_OK;
 }
 
-// Waits on a barrier nobody arrives on, with the kernels' own bounded wait but a short limit, and
-// reports the give-up the way they do (status word 0 = 1, word 1 = the site).
+// Waits on a barrier nobody arrives on, then on a flag nobody sets (a status word that stays zero), with the kernels' own
+// bounded waits but a short limit, and reports that both gave up the way they do (status word 0 = 1, word 1 = the site).
 __global__ void atf_bounded_wait_selftest_kernel(unsigned int* status, unsigned long long limit_ns) {
   __shared__ alignas(8) unsigned long long barmem;
   const uint32_t bar = smem_u32(&barmem);
@@ -115,7 +115,7 @@ __global__ void atf_bounded_wait_selftest_kernel(unsigned int* status, unsigned 
 #pragma unroll 1
       for (int i = 0; i < 64 && !done; ++i) done = mbar_try_wait(bar, 0);
     }
-    if (!done) {
+    if (!done && flag_wait(status + 2, limit_ns) == 0u) {
       atomicExch(status, 1u);
       atomicExch(status + 1, 99u);
     }

@@ -280,12 +280,10 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   if (CUT && second && cut > 0) {
     if (tid == 0) {
       grid_dependency_wait();
-      const unsigned long long w0 = global_timer_ns();
-      unsigned int f;
-      while ((f = ld_acquire(P.flags + ((int)blockIdx.x - P.jobs))) == 0u && global_timer_ns() - w0 <= ATF_WAIT_LIMIT_NS) __nanosleep(200);
+      const unsigned int f = flag_wait(P.flags + ((int)blockIdx.x - P.jobs), ATF_WAIT_LIMIT_NS);
       if (f == 0u) {
         s_abort = 1;
-        fail_site = 40;
+        fail_site = 38;
       }
       if (f == 2u) {
         s_redo = 1;

@@ -67,12 +67,7 @@ __device__ __forceinline__ uint32_t ld_sched(const uint32_t* p) {
   return w;
 }
 
-// The flag between the two blocks of a cut tile.
-__device__ __forceinline__ unsigned int ld_acquire(const unsigned int* p) {
-  unsigned int v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
+// The flag between the two blocks of a cut tile (flag_wait reads it).
 __device__ __forceinline__ void st_release(unsigned int* p, unsigned int v) {
   asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }

@@ -66,3 +66,12 @@ def test_sums_are_read_behind_a_barrier_of_the_warp():
     wait = body.index("bar(B_PFULL + 2 * sb + h)")
     between = body[body.index("__shfl_sync", wait):body.index("lds_f4(", wait)]
     assert "__syncwarp();" in between
+
+
+def test_a_give_up_names_its_kernel():
+    """Prefill and decode report in the same status word: no two files share the code of a wait."""
+    used = {}
+    for f in sorted(os.listdir(CSRC)):
+        for site in re.findall(r"fail_site = (\d+);|atomicExch\(status \+ 1, (\d+)u\)", open(os.path.join(CSRC, f)).read()):
+            used.setdefault(int(site[0] or site[1]), set()).add(f)
+    assert used.pop(0) and len(used) > 10 and all(len(files) == 1 for files in used.values()), used
