@@ -13,10 +13,15 @@
 // host side
 // ------------------------------------------------------------------------------------------
 atf_status atf_fail(atf_status code, const char* fmt, ...);
+// An error that a call returned also stays the runtime's last error, which the next ordinary launch's check would report as its
+// own: it is taken from there, too.
 #define ATF_CUDA_CHECK(expr)                                                              \
   do {                                                                                    \
     cudaError_t _e = (expr);                                                              \
-    if (_e != cudaSuccess) return atf_fail(ATF_ERR_CUDA, "%s: %s", #expr, cudaGetErrorString(_e)); \
+    if (_e != cudaSuccess) {                                                              \
+      (void)cudaGetLastError();                                                           \
+      return atf_fail(ATF_ERR_CUDA, "%s: %s", #expr, cudaGetErrorString(_e));             \
+    }                                                                                     \
   } while (0)
 
 constexpr int ATF_MAX_PAIRS = 64;  // d <= 128

@@ -958,7 +958,6 @@ atf_status launch_decode(const DecodeParams& P, const AtfTable& t, int B, int mo
     if (count) ATF_DEC_LAUNCH(ATF_MODE_COARSE, true); else ATF_DEC_LAUNCH(ATF_MODE_COARSE, false);
   }
 #undef ATF_DEC_LAUNCH
-  ATF_CUDA_CHECK(cudaGetLastError());
   return ATF_OK;
 }
 
@@ -982,7 +981,6 @@ atf_status launch_decode_tiles(const CUtensorMap& tmV, const DecodeParams& P, co
     if (count) ATF_TL_LAUNCH(ATF_MODE_COARSE, true); else ATF_TL_LAUNCH(ATF_MODE_COARSE, false);
   }
 #undef ATF_TL_LAUNCH
-  ATF_CUDA_CHECK(cudaGetLastError());
   return ATF_OK;
 }
 

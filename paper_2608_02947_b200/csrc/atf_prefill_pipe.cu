@@ -991,7 +991,6 @@ atf_status launch_pipe(const CUtensorMap& tq, const CUtensorMap& tql, const CUte
     ATF_PP_LAUNCH(ATF_MODE_COARSE, false, false);
   }
 #undef ATF_PP_LAUNCH
-  ATF_CUDA_CHECK(cudaGetLastError());
   return ATF_OK;
 }
 

@@ -69,3 +69,40 @@ def test_every_window_covering_the_prompt_makes_all_modes_one(atf):
         outs.append((O.clone(), LSE.clone()))
     for O, LSE in outs[1:]:
         assert torch.equal(O.view(torch.int16), outs[0][0].view(torch.int16)) and torch.equal(LSE, outs[0][1])
+
+
+@pytest.mark.parametrize("call", ["rope", "decode", "prefill"])
+def test_a_failed_launch_is_reported_once(atf, call):
+    """A launch into a capture that has been invalidated (by a synchronisation) is refused by the runtime; the next call, on a
+    stream that captures nothing, must not report that error again."""
+    import ctypes as C
+    X = torch.ones((1, 2, 300, 64), dtype=torch.bfloat16, device="cuda")
+    _, theta = atf.atf_window_table(1e6, 64, 2.0, 300)
+    calls = {"rope": lambda: atf.atf_rope(X.clone(), theta), "decode": lambda: atf.atf_decode(X[:, :, -1].contiguous(), X, X),
+             "prefill": lambda: atf.atf_prefill(X, X, X)}
+    calls[call]()
+    torch.cuda.synchronize()
+    q, O, lse = X[:, :, -1].contiguous(), torch.empty_like(X), torch.empty((1, 2, 300), device="cuda")
+    in_capture = {"rope": lambda: atf.atf_rope(O, theta), "decode": lambda: atf.atf_decode(q, X, X, O=q),
+                  "prefill": lambda: atf.atf_prefill(X, X, X, O=O, LSE=lse)}[call]
+    rt = C.CDLL("libcudart.so.12")
+    rt.cudaStreamBeginCapture.argtypes = [C.c_void_p, C.c_int]
+    rt.cudaStreamSynchronize.argtypes = [C.c_void_p]
+    rt.cudaStreamEndCapture.argtypes = [C.c_void_p, C.c_void_p]
+    stream, graph = torch.cuda.Stream(), C.c_void_p()
+    with torch.cuda.stream(stream):
+        assert rt.cudaStreamBeginCapture(stream.cuda_stream, 2) == 0  # relaxed
+        refused = rt.cudaStreamSynchronize(stream.cuda_stream)
+        try:
+            with pytest.raises(atf.AtfError) as e:
+                in_capture()
+        finally:
+            ended = rt.cudaStreamEndCapture(stream.cuda_stream, C.byref(graph))
+            rt.cudaGetLastError()
+    assert refused != 0 and ended != 0 and e.value.code == 3
+    cache = atf.atf_kcache_pack(X)
+    torch.cuda.synchronize()
+    assert int(cache.float().sum()) == X.numel()
+    calls[call]()
+    torch.cuda.synchronize()
+    atf.binding.check_status()
