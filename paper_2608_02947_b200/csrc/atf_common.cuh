@@ -161,13 +161,17 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
   }
 }
 
-// Bounded wait for a word that another block sets with a release: its value, 0 if it was still 0 after limit_ns.
-__device__ __forceinline__ unsigned int flag_wait(const unsigned int* flag, unsigned long long limit_ns) {
+// A word that another block sets, and a bounded wait until one of its bits in `mask` is set: the word as last seen.
+__device__ __forceinline__ unsigned int ld_acquire(const unsigned int* p) {
+  unsigned int v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ unsigned int flag_wait(const unsigned int* flag, unsigned int mask, unsigned long long limit_ns) {
   const unsigned long long t0 = global_timer_ns();
   for (;;) {
-    unsigned int v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(flag) : "memory");
-    if (v != 0u || global_timer_ns() - t0 > limit_ns) return v;
+    const unsigned int v = ld_acquire(flag);
+    if ((v & mask) != 0u || global_timer_ns() - t0 > limit_ns) return v;
     __nanosleep(200);
   }
 }

@@ -115,7 +115,7 @@ __global__ void atf_bounded_wait_selftest_kernel(unsigned int* status, unsigned 
 #pragma unroll 1
       for (int i = 0; i < 64 && !done; ++i) done = mbar_try_wait(bar, 0);
     }
-    if (!done && flag_wait(status + 2, limit_ns) == 0u) {
+    if (!done && flag_wait(status + 2, ~0u, limit_ns) == 0u) {
       atomicExch(status, 1u);
       atomicExch(status + 1, 99u);
     }

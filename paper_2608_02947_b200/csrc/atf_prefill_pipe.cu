@@ -206,8 +206,8 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int n0 = P.N - P.Nq;
-  // Blocks start in the order of their index: the tiles of a group of heads, longest rows first.  CUT: the first P.cuts tiles
-  // are worked on by two blocks (atf_prefill_cuts).
+  // The tiles of a group of heads, longest rows first (blocks start about in the order of their index).  CUT: the first P.cuts
+  // tiles are worked on by two blocks (atf_prefill_cuts).
   const int ntq = (P.N + T - 1) / T;
   const bool first = CUT && (int)blockIdx.x < P.cuts, second = CUT && (int)blockIdx.x >= P.jobs;
   const int job = second ? (int)blockIdx.x - P.jobs : (int)blockIdx.x;
@@ -271,8 +271,8 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   volatile int* abortp = &s_abort;
   unsigned int fail_site = 0;
 
-  // A cut tile's state: O (fp32, [D / 4][128 rows][4]), the sums of the two key halves, the rows' reference; and a flag (1: there,
-  // 2: a sum has overflowed, the whole tile takes the safe form).
+  // A cut tile's state: O (fp32, [D / 4][128 rows][4]), the sums of the two key halves, the rows' reference; and a flag (with
+  // CUT_OVERFLOW a sum has overflowed: the whole tile takes the safe form).
   auto cut_state = [&]() {
     const int j = (int)blockIdx.x < P.cuts ? (int)blockIdx.x : (int)blockIdx.x - P.jobs;
     return P.state + (int64_t)j * (T * (D + 3));
@@ -280,14 +280,19 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   if (CUT && second && cut > 0) {
     if (tid == 0) {
       grid_dependency_wait();
-      const unsigned int f = flag_wait(P.flags + ((int)blockIdx.x - P.jobs), ATF_WAIT_LIMIT_NS);
-      if (f == 0u) {
-        s_abort = 1;
-        fail_site = 38;
-      }
-      if (f == 2u) {
-        s_redo = 1;
-        s_part[0] = nt;  // no step of the fast pass
+      const unsigned int* flag = P.flags + ((int)blockIdx.x - P.jobs);
+      if (ld_acquire(flag) == 0u) {
+        s_part[0] = 0;  // the first block has not started: the whole tile
+      } else {
+        const unsigned int f = flag_wait(flag, CUT_STATE_THERE, ATF_WAIT_LIMIT_NS);
+        if (!(f & CUT_STATE_THERE)) {
+          s_abort = 1;
+          fail_site = 38;
+        }
+        if (f & CUT_OVERFLOW) {
+          s_redo = 1;
+          s_part[0] = nt;  // no step of the fast pass
+        }
       }
     }
     __syncthreads();
@@ -449,6 +454,10 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     }
   } else if (warp == 3) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+    if (first) {
+      grid_dependency_wait();  // the pre-pass zeroes the flags
+      if (lane == 0) st_release(P.flags + blockIdx.x, CUT_RUNS);
+    }
     for (int pass = 0; pass < 2; ++pass)
       if (!another_pass(pass)) break;
   } else {
@@ -931,7 +940,7 @@ atf_prefill_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   }
   tc_fence_before();
   __syncthreads();
-  if (CUT && tid == 0 && s_part[CUT ? 1 : 0] && !s_abort) st_release(P.flags + blockIdx.x, s_redo ? 2u : 1u);
+  if (CUT && tid == 0 && s_part[CUT ? 1 : 0] && !s_abort) st_release(P.flags + blockIdx.x, CUT_RUNS | CUT_STATE_THERE | (s_redo ? CUT_OVERFLOW : 0));
   if (warp == 0) tmem_dealloc(tmem_base, TMEM_COLS);
 }
 

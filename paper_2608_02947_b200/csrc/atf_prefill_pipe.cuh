@@ -39,8 +39,10 @@ constexpr int ATF_PREP_THREADS = 256;
 // 24 heads are 5.2 waves that run as 6).  Then the first ATF_SMS tiles are worked on by two blocks each: blocks 0 .. ATF_SMS - 1
 // take the first (j + 1/2) / ATF_SMS of tile j's steps, which lets the SMs fall out of step evenly, and the blocks behind all
 // others go on where those stopped, the longest rest first, so that all SMs end together.  O, row sums and reference pass
-// through memory in fp32 as they stand: the result is bit for bit that of one block.  A block waits for one that started
-// before it, at a time when that one is long done.
+// through memory in fp32 as they stand: the result is bit for bit that of one block.  The second block of a
+// tile comes at a time when the first is long done.  CUDA promises no order in which blocks start, though, so it waits only for a
+// first block that has said that it runs (and waits for no other block itself); if that one has not started, the second takes the
+// whole tile, and what the first one does later is read by nobody.
 // Cut where the idle share is above a fifth: the kernel with the cut is 2 to 4 % slower, rows out of step share fewer K and V
 // tiles in L2, and under the power cap idle SMs leave their power to the others (us, whole -> cut: 2000 of 20000, 14 heads of 64,
 // 24 % idle, exact 274 -> 250, coarse 226 -> 211; 24 heads of 128, 1000 of 12000, 37 %, 222 -> 208, 1000 of 100000, full, 37 %,
@@ -67,7 +69,8 @@ __device__ __forceinline__ uint32_t ld_sched(const uint32_t* p) {
   return w;
 }
 
-// The flag between the two blocks of a cut tile (flag_wait reads it).
+// The flag between the two blocks of a cut tile, written by the first one.
+enum { CUT_RUNS = 1, CUT_STATE_THERE = 2, CUT_OVERFLOW = 4 };
 __device__ __forceinline__ void st_release(unsigned int* p, unsigned int v) {
   asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }

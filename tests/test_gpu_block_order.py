@@ -3,6 +3,16 @@ import pytest
 import torch
 
 pytestmark = pytest.mark.gpu
+SMS = 148  # tiles that are cut, if any
+
+
+def _cut_flags(ws, B, Hq, Hkv, N, Nq, d, split=False):
+    """The flags of the cut tiles, in the workspace behind schedule, operands and state."""
+    part = lambda heads, rows: (B * heads * rows * d * 2 + 255) // 256 * 256
+    at = 256 + 4 * 16384 + (((N + 127) // 128 + 1) * 32 + 255) // 256 * 256
+    at += 2 * (part(Hq, Nq) + part(Hkv, N)) if split else part(Hkv, N)
+    at += SMS * 128 * (d + 3) * 4
+    return ws[at:at + 4 * SMS].view(torch.int32)
 
 
 # rows of different lengths; keys and values of a KV head: 36 MB (one a group), 13 MB (two groups, the last one short); split
@@ -50,4 +60,25 @@ def test_cut_tiles(B, Hq, Hkv, N, Nq, d, mode, far, split):
     for _ in range(3):
         O, lse = call(Q, K, V, table=W, mode=mode)
         assert torch.equal(O, whole[0]) and torch.equal(lse, whole[1])
+    atf.binding.check_status()
+
+
+# CUDA promises no order in which blocks start: the second block of a cut tile waits only for a first one that runs.  Every first
+# block with a part has said so (1) and that its state is there (2).
+@pytest.mark.parametrize("B,Hq,Hkv,N,Nq,d,mode,split", [(1, 24, 8, 9000, 850, 128, 0, False), (2, 14, 2, 12345, 700, 64, 1, False),
+                                                        (1, 24, 8, 9000, 850, 128, 0, True)])
+def test_first_blocks_of_cut_tiles_say_that_they_run(B, Hq, Hkv, N, Nq, d, mode, split):
+    import paper_2608_02947_b200 as atf
+    kind = torch.float32 if split else torch.bfloat16
+    Q, K, V = [torch.randn((B, h, n, d), device="cuda").to(t) for h, n, t in ((Hq, Nq, kind), (Hkv, N, kind), (Hkv, N, torch.bfloat16))]
+    W, _ = atf.atf_window_table(5e5, d, 2.0, N)
+    ws = atf.ensure_workspace(3 * atf.atf_workspace_bytes(atf.binding.ATF_OP_PREFILL_SPLIT, B, Hq, Hkv, N, d), "cuda:0")
+    flags = _cut_flags(ws, B, Hq, Hkv, N, Nq, d, split)
+    for _ in range(2):  # the second call finds what the first one left
+        flags.fill_(-1)
+        (atf.atf_prefill_split if split else atf.atf_prefill)(Q, K, V, table=W, mode=mode)
+        torch.cuda.synchronize()
+        got = flags.tolist()
+        steps = [min((N - 1) // 128 - j // (B * Hq) + 1, (int(W.max()) + 127) // 128 + 1) for j in range(SMS)]
+        assert got == [3 if n * (2 * j + 1) // (2 * SMS) else 0 for j, n in enumerate(steps)]
     atf.binding.check_status()
