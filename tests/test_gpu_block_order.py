@@ -35,13 +35,7 @@ def test_heads_in_groups(B, Hq, Hkv, N, Nq, d, split):
     atf.binding.check_status()
 
 
-# Bit for bit what one block gives (a call that counts terms never cuts): just above one wave of blocks, an odd number of waves,
-# ragged rows, windows that end (equal short tiles), the safe second pass seen in front of the cut and behind it, the split form
-@pytest.mark.parametrize("B,Hq,Hkv,N,Nq,d,mode,far,split", [
-    (1, 24, 8, 9000, 850, 128, 0, 0, False), (2, 14, 2, 12345, 700, 64, 0, 0, False), (1, 24, 8, 30000, 1111, 128, 1, 0, False),
-    (1, 40, 8, 9000, 512, 128, 0, 1, False), (1, 40, 8, 9000, 512, 64, 0, 2, False), (1, 40, 8, 9000, 512, 128, 1, 2, False),
-    (3, 14, 2, 20000, 500, 64, 1, 3, False), (1, 24, 8, 9000, 850, 128, 0, 0, True), (1, 40, 8, 9000, 512, 128, 0, 2, True)])
-def test_cut_tiles(B, Hq, Hkv, N, Nq, d, mode, far, split):
+def _cut_case(B, Hq, Hkv, N, Nq, d, far, split):
     import paper_2608_02947_b200 as atf
     g = torch.Generator(device="cuda").manual_seed(N + far)
     kind = torch.float32 if split else torch.bfloat16
@@ -49,18 +43,57 @@ def test_cut_tiles(B, Hq, Hkv, N, Nq, d, mode, far, split):
     W, _ = atf.atf_window_table(5e5, d, 2.0, N)
     if far == 3:  # no pair reaches further: every tile has the same few steps
         W = W.clamp(max=7000)
+    elif far == 4:  # every pair reaches every key
+        W = None
     elif far:     # logits that the reference of the diagonal tile cannot hold, in near (1) or far (2) keys
         K[:, :, slice(N - 2000, N - 1500) if far == 1 else slice(0, 500)] *= 30
         Q *= 4
-    Q, K, V = Q.to(kind), K.to(kind), V.to(torch.bfloat16)
+    return Q.to(kind), K.to(kind), V.to(torch.bfloat16), W
+
+
+# Bit for bit what one block gives (a call that counts terms never cuts): just above one wave of blocks, an odd number of waves,
+# ragged rows, windows that end (equal short tiles), the safe second pass seen in front of the cut and behind it; every form of the
+# kernel goes on from a state.  The third case lies just below the idle share from which tiles are cut.
+@pytest.mark.parametrize("B,Hq,Hkv,N,Nq,d,mode,far,split", [
+    (1, 24, 8, 9000, 850, 128, 0, 0, False), (2, 14, 2, 12345, 700, 64, 0, 0, False), (1, 24, 8, 30000, 1111, 128, 1, 0, False),
+    (1, 40, 8, 9000, 512, 128, 0, 1, False), (1, 40, 8, 9000, 512, 64, 0, 2, False), (1, 40, 8, 9000, 512, 128, 1, 2, False),
+    (3, 14, 2, 20000, 500, 64, 1, 3, False), (1, 24, 8, 9000, 850, 128, 0, 0, True), (1, 40, 8, 9000, 512, 128, 0, 2, True),
+    (1, 24, 8, 9000, 850, 128, 1, 0, False), (1, 24, 8, 9000, 850, 128, 0, 4, False), (2, 14, 2, 12345, 700, 64, 0, 4, False),
+    (1, 40, 8, 9000, 512, 128, 1, 1, False), (1, 24, 8, 9000, 850, 128, 1, 0, True), (2, 14, 2, 12345, 700, 64, 0, 0, True),
+    (2, 14, 2, 12345, 700, 64, 1, 1, True)])
+def test_cut_tiles(B, Hq, Hkv, N, Nq, d, mode, far, split):
+    import paper_2608_02947_b200 as atf
+    Q, K, V, W = _cut_case(B, Hq, Hkv, N, Nq, d, far, split)
     call = atf.atf_prefill_split if split else atf.atf_prefill
     # room for the state of the cut tiles beside what the call asks for
-    atf.ensure_workspace(3 * atf.atf_workspace_bytes(atf.binding.ATF_OP_PREFILL, B, Hq, Hkv, N, d), "cuda:0")
+    ws = atf.ensure_workspace(3 * atf.atf_workspace_bytes(atf.binding.ATF_OP_PREFILL_SPLIT, B, Hq, Hkv, N, d), "cuda:0")
+    flags = _cut_flags(ws, B, Hq, Hkv, N, Nq, d, split)
     whole = call(Q, K, V, table=W, mode=mode, kept_terms=torch.zeros(B * Hq, dtype=torch.int64, device="cuda"))
     for _ in range(3):
+        flags.fill_(-1)
         O, lse = call(Q, K, V, table=W, mode=mode)
         assert torch.equal(O, whole[0]) and torch.equal(lse, whole[1])
+        seen = flags.tolist()
+        if N == 30000:
+            assert set(seen) == {-1}
+        else:  # 3: went on from the state; 7: overflow in the first part, all of it again; 0: no first part
+            assert set(seen) <= ({0, 3, 7} if far in (1, 2) else {0, 3})
+            assert seen.count(3) > (10 if far == 1 else 100) and (far != 1 or seen.count(7) > 50)
     atf.binding.check_status()
+
+
+@pytest.mark.parametrize("d,mode,far", [(128, 0, 0), (128, 1, 1), (64, 0, 1), (64, 1, 0)])
+def test_cut_output_over_its_queries(d, mode, far):
+    import paper_2608_02947_b200 as atf
+    B, Hq, Hkv, N, Nq = 1, 40, 8, 9000, 512
+    Q, K, V, W = _cut_case(B, Hq, Hkv, N, Nq, d, far, False)
+    ws = atf.ensure_workspace(3 * atf.atf_workspace_bytes(atf.binding.ATF_OP_PREFILL, B, Hq, Hkv, N, d), "cuda:0")
+    flags = _cut_flags(ws, B, Hq, Hkv, N, Nq, d)
+    O, lse = atf.atf_prefill(Q, K, V, table=W, mode=mode)
+    flags.fill_(-1)
+    got, lse2 = atf.atf_prefill(Q, K, V, table=W, mode=mode, O=Q)
+    assert got.data_ptr() == Q.data_ptr() and torch.equal(got, O) and torch.equal(lse2, lse)
+    assert 3 in flags.tolist()
 
 
 # CUDA promises no order in which blocks start: the second block of a cut tile waits only for a first one that runs.  Every first
