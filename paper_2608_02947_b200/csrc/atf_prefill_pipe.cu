@@ -954,16 +954,24 @@ atf_status launch_pipe(const CUtensorMap& tq, const CUtensorMap& tql, const CUte
   attr.val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg = {};
   // Order of the tiles.  Rows of different lengths: longest first over all heads, so that no head's longest row starts when the
-  // others are done (us, head by head -> so: a layer step of 24 heads x 8192 rows 642 -> 634, 3000 rows 172 -> 141, 14 heads x
-  // 1200 of 64 26.4 -> 21.3), in equal groups of heads whose K and V stay in L2 together.  Rows of about the same length: head
-  // by head (B = 2, 24 heads, 2048 rows of 8192: 457, over all heads 470; 2 x 2 heads, 16000 of 60000: 1226 against 1265).
+  // others are done (us, head by head -> so: 24 heads x 8192 rows 596 -> 581, 3000 rows 174 -> 141, 3500 of 5000 277 -> 250, 14
+  // heads x 5000 of 8000, d = 64, 224 -> 200).  Rows of about the same length: head by head (2048 rows of 16384 403, over all
+  // heads 418; B = 2, 4096 of 8192 778, 795; 2 x 2 heads, 16000 of 60000 1226, 1264; but 14 heads, 6000 of 20000, 599, 589).  Head by
+  // head, too, where a head has tiles for half the SMs, so that it alone comes near a sorted wave, and longest first would leave the
+  // last wave, of the shortest rows, idle for more than a quarter of a mean tile (2 x 2 heads: 14700 of 25000, last wave 0.14 full, 430
+  // against 451, 16384 of 31955, 0.49, 580, 612; 13100 of 22277, 0.81, 354 against 340: longest first; 14 heads: 8000 of 13607, 64
+  // tiles, 0.05, 490, 501, 16384 of 31955, 0.20, 1969, 2015; 14700 of 25000, 0.97, 1378, 1349: longest first; fewer tiles: 1664 of 2605,
+  // 24 heads, 0.27, 129, 109, 3200 of 5935, B = 2, 0.43, 541, 524: longest first).
+  // Groups of heads whose K and V take up to 64 MB together, because what all SMs read at a time is to stay in L2: 24 heads x 131072 rows
+  // 85.0 ms, in groups of 128 MB 85.5, over all heads 88.8.  32 to 48 MB are within 1.5 % of 64 (7000 to 131072 rows, 39 shapes).
   const int64_t dlim = ((int64_t)t.w[D / 2 - 1] + T - 1) / T + 1, per_kv = P.Hq / P.Hkv;
   const int64_t longest = std::min<int64_t>((P.N + T - 1) / T, dlim), shortest = std::min<int64_t>((P.N - P.Nq) / T + 1, dlim);
   P.heads = P.Hq * B;
+  const int64_t rest = ATF_SMS - 1 - ((int64_t)tiles * P.heads - 1) % ATF_SMS;  // blocks that the last wave lacks
   int64_t group = 1;
   if (P.cuts) {
     group = P.heads;
-  } else if (2 * shortest <= longest) {
+  } else if (2 * shortest <= longest && (tiles < 64 || 8 * rest * shortest <= ATF_SMS * (longest + shortest))) {
     const int64_t fit = std::max<int64_t>(1, (64ll << 20) / ((int64_t)P.N * D * 2 * (SPLIT ? 3 : 2))) * per_kv;
     const int64_t groups = (P.heads + fit - 1) / fit;
     group = std::min<int64_t>(((P.heads + groups - 1) / groups + per_kv - 1) / per_kv * per_kv, P.heads);
@@ -986,10 +994,11 @@ atf_status launch_pipe(const CUtensorMap& tq, const CUtensorMap& tql, const CUte
     ATF_CUDA_CHECK(cudaLaunchKernelEx(&cfg, kern, tq, tql, tk, tkl, tv, P, t));                        \
   } while (0)
   // In turns or in step: the results are the same, bit for bit.  In turns pays where the softmax holds the pace and no warp has
-  // cells to finish (us, in step -> in turns: coarse, 24 heads of 128, 8192 rows 446 -> 410, 32768 5780 -> 5210, 4000 of 61003
-  // 2650 -> 2415; 14 heads of 64, 32768 rows, coarse 2636 -> 2400, full 2520 -> 2290).  Full attention at d = 128 and the split-
-  // precision form are bound by the tensor pipe (8192 rows, full 432 -> 449); exact mode's finish is slower by one warp for all
-  // 128 keys (8192 rows 596 -> 690), and a kernel with both forms of it slower in either; calls that count terms stay in step.
+  // cells to finish (us, in step -> in turns: coarse, 24 heads of 128, 8192 rows 415 -> 397, 32768 5595 -> 5105, 131072 81.3 -> 78.0 ms,
+  // 4000 of 61003 2596 -> 2413; 14 heads of 64, 4096 rows, coarse 59.2 -> 57.4, 32768 rows 2539 -> 2381, full 2718 -> 2518).  Full
+  // attention at d = 128 is bound by the tensor pipe: the same either way up to 4096 rows, above that 1 to 2 % less in turns, inside the
+  // spread of one side's runs (8192 rows 433, 426; 32768 5760, 5700); so is the split-precision form, whose operands leave no room for a
+  // second exchange area.  Exact mode's finish is slower by one warp for all 128 keys (8192 rows 596 -> 690), and a kernel with both forms of it slower in either; calls that count terms stay in step.
   if (mode == ATF_MODE_EXACT) {
     if (count) ATF_PP_LAUNCH(ATF_MODE_EXACT, true, false); else ATF_PP_LAUNCH(ATF_MODE_EXACT, false, false);
   } else if (count) {

@@ -15,16 +15,33 @@ def _cut_flags(ws, B, Hq, Hkv, N, Nq, d, split=False):
     return ws[at:at + 4 * SMS].view(torch.int32)
 
 
+def _group(B, Hq, Hkv, N, Nq, d, split, W):
+    """Heads whose tiles are dealt out together, longest rows first, by the rule beside the launch; 1: head by head."""
+    tiles = (N + 127) // 128 - (N - Nq) // 128
+    reach = (int(W.max()) + 127) // 128 + 1
+    longest, shortest = min((N + 127) // 128, reach), min((N - Nq) // 128 + 1, reach)
+    if 2 * shortest > longest or (tiles >= 64 and 8 * (-tiles * B * Hq % SMS) * shortest > SMS * (longest + shortest)):
+        return 1
+    per_kv = Hq // Hkv
+    groups = -(-B * Hq // (max(1, (64 << 20) // (N * d * 2 * (3 if split else 2))) * per_kv))
+    return min(-(-(-(-B * Hq // groups)) // per_kv) * per_kv, B * Hq)
+
+
 # rows of different lengths; keys and values of a KV head: 36 MB (one a group), 13 MB (two groups, the last one short); split
-# mode: 27 MB (two groups, the last one short); rows of about the same length: head by head
-@pytest.mark.parametrize("B,Hq,Hkv,N,Nq,d,split", [(3, 6, 2, 70000, 36000, 128, False), (7, 2, 1, 50000, 26000, 64, False),
-                                                   (3, 3, 1, 35000, 18000, 128, True), (2, 6, 2, 9000, 300, 128, False)])
-def test_heads_in_groups(B, Hq, Hkv, N, Nq, d, split):
+# mode: 27 MB (two groups, the last one short); rows of about the same length: head by head; so, too, where a head has many tiles
+# and the last wave is not full, the first two against the next two; the last two lie on either side of 64 tiles
+@pytest.mark.parametrize("B,Hq,Hkv,N,Nq,d,split,group", [
+    (3, 6, 2, 70000, 36000, 128, False, 1), (7, 2, 1, 50000, 26000, 64, False, 1),
+    (3, 6, 2, 70000, 35696, 128, False, 3), (7, 2, 1, 50000, 26960, 64, False, 8),
+    (3, 3, 1, 35000, 18000, 128, True, 6), (2, 6, 2, 9000, 300, 128, False, 1),
+    (1, 14, 2, 13607, 8000, 64, False, 1), (1, 14, 2, 13600, 7900, 64, False, 14)])
+def test_heads_in_groups(B, Hq, Hkv, N, Nq, d, split, group):
     import paper_2608_02947_b200 as atf
     g = torch.Generator(device="cuda").manual_seed(N)
     kind = torch.float32 if split else torch.bfloat16
     Q, K, V = [torch.randn((B, h, n, d), generator=g, device="cuda").to(t) for h, n, t in ((Hq, Nq, kind), (Hkv, N, kind), (Hkv, N, torch.bfloat16))]
     W, _ = atf.atf_window_table(5e5, d, 2.0, N)
+    assert _group(B, Hq, Hkv, N, Nq, d, split, W) == group
     call = atf.atf_prefill_split if split else atf.atf_prefill
     O, lse = call(Q, K, V, table=W)
     for b in range(B):
