@@ -309,7 +309,9 @@ atf_status atf_decode_static(const void* q, const void* Kcache, const void* Vcac
  * process that drives several GPUs passes each call its own workspace in atf_opts.workspace.
  * A workspace sized for the largest call
  * serves prefill and decode in turn: its first 64.25 KiB (status words and decode's split
- * counters, which the kernels leave zeroed) are never used as scratch.  One call at a time may use a given
+ * counters, which the kernels leave zeroed) are never used as scratch; all behind that may be.  Where the last blocks of a
+ * prefill would leave the GPU idle, two blocks share a tile if the workspace has room for what passes between them: the size
+ * for N keys has from B Hq N = 40000 on; with less the call takes longer, with the same bits.  One call at a time may use a given
  * workspace; calls that overlap on the GPU need separate workspaces (atf_opts.workspace).     */
 enum { ATF_OP_PREFILL = 0, ATF_OP_DECODE = 1, ATF_OP_PREFILL_SPLIT = 2 };
 size_t atf_workspace_bytes(int op, int B, int Hq, int Hkv, int64_t N, int d);

@@ -82,7 +82,9 @@ atf_status atf_validate_table(const char* who, const int64_t* table, int d, int6
 static int sched_entries(int64_t N) { return (int)((N + T - 1) / T) + 1; }
 static size_t sched_bytes(int64_t N) { return ((size_t)sched_entries(N) * 32 + 255) & ~(size_t)255; }
 
-// Counts room for a reordered Q, which an earlier form of the pre-pass wrote: callers' sizes stay what they were.
+// Counts room for a reordered Q, which an earlier form of the pre-pass wrote: callers' sizes stay what they were.  What a workspace
+// has behind schedule and K, this room or more, holds the state of cut tiles: with less than that state takes a call is not cut
+// (atf_prefill_cuts; from B Hq N = 40000 on the size asked for here is enough).
 size_t atf_prefill_workspace_bytes(int B, int Hq, int Hkv, int64_t N, int d) {
   return ATF_WS_HEADER + sched_bytes(N) + repack_bytes(B, Hq, N, d) + repack_bytes(B, Hkv, N, d);
 }

@@ -44,9 +44,12 @@ constexpr int ATF_PREP_THREADS = 256;
 // first block that has said that it runs (and waits for no other block itself); if that one has not started, the second takes the
 // whole tile, and what the first one does later is read by nobody.
 // Cut where the idle share is above a fifth: the kernel with the cut is 2 to 4 % slower, rows out of step share fewer K and V
-// tiles in L2, and under the power cap idle SMs leave their power to the others (us, whole -> cut: 2000 of 20000, 14 heads of 64,
-// 24 % idle, exact 274 -> 250, coarse 226 -> 211; 24 heads of 128, 1000 of 12000, 37 %, 222 -> 208, 1000 of 100000, full, 37 %,
-// 1601 -> 1343; but 4000 of 61003, coarse, 15 %, 2510 -> 2516).
+// tiles in L2, and under the power cap idle SMs leave their power to the others (us, whole -> cut: 24 heads of 128, 850 of 9000, 52 %
+// idle, exact 189 -> 170, coarse 125 -> 102, 1000 of 12000, 35 %, 225 -> 208, 1000 of 100000, full, 37 %, 1660 -> 1308; 14 heads of 64,
+// 1600 of 20000, 49 %, 229 -> 177; 24 heads, 900 of 2600, 45 %, 99.7 -> 100.3).  Not cut: 2000 of 40000, 9 %, 1020 -> 1078, 1400 of
+// 40000, 3 %, 704 -> 783, 4000 of 61003, 15 %, exact 2880 -> 2960, coarse 2750 -> 2660.  The twelve steps an SM beside the fifth stand
+// for what a cut costs whatever the length; between 20 and 25 % they refuse calls on both sides: 3000 of 20000, 21 %, 809 -> 817, but
+// 1111 of 30000, 23 %, 512 -> 476, and 14 heads of 64, 2000 of 20000, 23 %, 274 -> 250.
 constexpr int ATF_SMS = 148;
 inline size_t atf_cut_floats(int d) { return (size_t)ATF_SMS * 128 * (d + 3); }
 inline int atf_prefill_cuts(int64_t N, int64_t Nq, int64_t heads, int w_max, int d, size_t spare_bytes) {
