@@ -964,6 +964,9 @@ atf_status launch_pipe(const CUtensorMap& tq, const CUtensorMap& tql, const CUte
   // 24 heads, 0.27, 129, 109, 3200 of 5935, B = 2, 0.43, 541, 524: longest first).
   // Groups of heads whose K and V take up to 64 MB together, because what all SMs read at a time is to stay in L2: 24 heads x 131072 rows
   // 85.0 ms, in groups of 128 MB 85.5, over all heads 88.8.  32 to 48 MB are within 1.5 % of 64 (7000 to 131072 rows, 39 shapes).
+  // Where one KV head's alone take more, head by head (28/4 heads of 128, full attention: 262144 rows 417, grouped 417 ms, 524288 1667,
+  // 1730, 1048576 6757, 8820, coarse 5675, 5840, exact 5935, 5915; in the slow one the power cap holds the clock at 945 MHz instead of
+  // 1410, presumably for K and V that come from DRAM again).
   const int64_t dlim = ((int64_t)t.w[D / 2 - 1] + T - 1) / T + 1, per_kv = P.Hq / P.Hkv;
   const int64_t longest = std::min<int64_t>((P.N + T - 1) / T, dlim), shortest = std::min<int64_t>((P.N - P.Nq) / T + 1, dlim);
   P.heads = P.Hq * B;
@@ -972,9 +975,11 @@ atf_status launch_pipe(const CUtensorMap& tq, const CUtensorMap& tql, const CUte
   if (P.cuts) {
     group = P.heads;
   } else if (2 * shortest <= longest && (tiles < 64 || 8 * rest * shortest <= ATF_SMS * (longest + shortest))) {
-    const int64_t fit = std::max<int64_t>(1, (64ll << 20) / ((int64_t)P.N * D * 2 * (SPLIT ? 3 : 2))) * per_kv;
-    const int64_t groups = (P.heads + fit - 1) / fit;
-    group = std::min<int64_t>(((P.heads + groups - 1) / groups + per_kv - 1) / per_kv * per_kv, P.heads);
+    const int64_t fit = (64ll << 20) / ((int64_t)P.N * D * 2 * (SPLIT ? 3 : 2)) * per_kv;
+    if (fit > 0) {
+      const int64_t groups = (P.heads + fit - 1) / fit;
+      group = std::min<int64_t>(((P.heads + groups - 1) / groups + per_kv - 1) / per_kv * per_kv, P.heads);
+    }
   }
   P.group = (int)std::max<int64_t>(group, (P.heads + 65534) / 65535);  // gridDim.y
   P.jobs = tiles * P.group;

@@ -23,18 +23,23 @@ def _group(B, Hq, Hkv, N, Nq, d, split, W):
     if 2 * shortest > longest or (tiles >= 64 and 8 * (-tiles * B * Hq % SMS) * shortest > SMS * (longest + shortest)):
         return 1
     per_kv = Hq // Hkv
-    groups = -(-B * Hq // (max(1, (64 << 20) // (N * d * 2 * (3 if split else 2))) * per_kv))
+    fit = (64 << 20) // (N * d * 2 * (3 if split else 2)) * per_kv
+    if fit == 0:
+        return 1
+    groups = -(-B * Hq // fit)
     return min(-(-(-(-B * Hq // groups)) // per_kv) * per_kv, B * Hq)
 
 
 # rows of different lengths; keys and values of a KV head: 36 MB (one a group), 13 MB (two groups, the last one short); split
 # mode: 27 MB (two groups, the last one short); rows of about the same length: head by head; so, too, where a head has many tiles
-# and the last wave is not full, the first two against the next two; the last two lie on either side of 64 tiles
+# and the last wave is not full, the first two against the next two; the next two lie on either side of 64 tiles,
+# the last two of 64 MB
 @pytest.mark.parametrize("B,Hq,Hkv,N,Nq,d,split,group", [
     (3, 6, 2, 70000, 36000, 128, False, 1), (7, 2, 1, 50000, 26000, 64, False, 1),
     (3, 6, 2, 70000, 35696, 128, False, 3), (7, 2, 1, 50000, 26960, 64, False, 8),
     (3, 3, 1, 35000, 18000, 128, True, 6), (2, 6, 2, 9000, 300, 128, False, 1),
-    (1, 14, 2, 13607, 8000, 64, False, 1), (1, 14, 2, 13600, 7900, 64, False, 14)])
+    (1, 14, 2, 13607, 8000, 64, False, 1), (1, 14, 2, 13600, 7900, 64, False, 14),
+    (1, 2, 1, 131072, 131072, 128, False, 2), (1, 2, 1, 131073, 131073, 128, False, 1)])
 def test_heads_in_groups(B, Hq, Hkv, N, Nq, d, split, group):
     import paper_2608_02947_b200 as atf
     g = torch.Generator(device="cuda").manual_seed(N)
