@@ -46,7 +46,7 @@ constexpr int ATF_PREP_THREADS = 256;
 // Cut where the idle share is above a fifth: the kernel with the cut is 2 to 4 % slower, rows out of step share fewer K and V
 // tiles in L2, and under the power cap idle SMs leave their power to the others (us, whole -> cut: 24 heads of 128, 850 of 9000, 52 %
 // idle, exact 189 -> 170, coarse 125 -> 102, 1000 of 12000, 35 %, 225 -> 208, 1000 of 100000, full, 37 %, 1660 -> 1308; 14 heads of 64,
-// 1600 of 20000, 49 %, 229 -> 177; 24 heads, 900 of 2600, 45 %, 99.7 -> 100.3).  Not cut: 2000 of 40000, 9 %, 1020 -> 1078, 1400 of
+// 1600 of 20000, 49 %, 229 -> 177; 28 heads of 128, 900 of 1000000, full, 17.0 -> 14.6 ms; 24 heads, 900 of 2600, 45 %, 99.7 -> 100.3 us).  Not cut: 2000 of 40000, 9 %, 1020 -> 1078, 1400 of
 // 40000, 3 %, 704 -> 783, 4000 of 61003, 15 %, exact 2880 -> 2960, coarse 2750 -> 2660.  The twelve steps an SM beside the fifth stand
 // for what a cut costs whatever the length; between 20 and 25 % they refuse calls on both sides: 3000 of 20000, 21 %, 809 -> 817, but
 // 1111 of 30000, 23 %, 512 -> 476, and 14 heads of 64, 2000 of 20000, 23 %, 274 -> 250.
